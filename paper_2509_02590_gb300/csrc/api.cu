@@ -336,7 +336,7 @@ void dump_item_profile(const RefineParams &p, const char *path, int ctas, cudaSt
   FILE *f = fopen(path, "a");
   if (!f) return;
   fprintf(f, "seq,n,E,nalive,passes,nsv,outcome,smid,slab,top,load,extract,ccr,peel,cc,contract,"
-             "sw,out,t_begin,t_end,p1_cycles,p1_marks,p1_steps,later_passes,forest,nsv1,forest_cycles,f_bfs,f_levels,f_check,"
+             "sw,out,t_begin,t_end,p1_cycles,p1_rounds,p1_phases,later_passes,forest,nsv1,forest_cycles,f_bfs,f_levels,f_check,"
              "f_trees,f_contract,f_relabel\n");
   for (const ItemProf &q : h)
     fprintf(f, "%u,%d,%d,%d,%d,%d,%d,%d,%d,%d,%u,%u,%u,%u,%u,%u,%u,%u,%lld,%lld,%lld,%lld,%lld,%lld,%d,%d,"

@@ -141,7 +141,7 @@ struct ItemProf {
   int n, E, nalive, passes, nsv, outcome, smid, slab, top;
   unsigned dt[8];
   long long t_begin, t_end;  // %globaltimer (ns) when the item started and ended
-  long long dbg[4];  // first contraction pass: loop cycles, pick cycles, steps, scan cycles
+  long long dbg[4];  // first contraction pass: cycles, rounds, phases; cycles of the later passes
   int forest;        // forest test: rounds it took (negative: gave up after that many)
   int nsv1;          // super-vertices after the first contraction pass
   long long forest_cycles;
