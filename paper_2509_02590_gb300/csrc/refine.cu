@@ -6,10 +6,10 @@
 // Per item (paper: Algorithm 1 for input clusters, then Algorithm 3 with a
 // peel and a connectivity check in front of the cut):
 //   1. extraction of the induced subgraph G[S] (Algorithm 1 / 3: E_c = edges
-//      with both ends in V_c) into a local CSR, local id = rank of the global
-//      id in S: one flat, load-balanced pass over all adjacency entries of
-//      the members with an 8-byte gather of slot[u] = (item << 32 | local id)
-//      per entry; local ids are 16-bit when the item has < 65535 vertices;
+//      with both ends in V_c) into local rows, local id = rank of the global
+//      id in S: one pass over all adjacency entries of the members with an
+//      8-byte gather of slot[u] = (item << 32 | local id) per entry; local
+//      ids are 16-bit when the item has < 65535 vertices;
 //   2. input clusters only: connected components (CCR); each component with
 //      at least min_size vertices is queued, or refinement continues in place
 //      when the cluster is one component;
@@ -45,6 +45,8 @@ constexpr size_t SMEM_MAX_BYTES = 227 * 1024;  // opt-in limit per CTA
 // generic ones.
 extern __shared__ __align__(16) char wcc_dyn_smem[];
 
+// Rows of more entries are extracted by all warps together.
+constexpr int LONG_ROW = 1024;
 // Most small input clusters a CTA claims at once (see k_refine).  With one per
 // warp and a barrier after them (a block of 7, 3.3 items a batch on average)
 // 2M vertices in 100,000 small clusters took 9.29 ms instead of 4.21.
@@ -69,6 +71,7 @@ __host__ __device__ inline size_t ws_bytes(int64_t n, int64_t d) {
   b += 3 * align16((size_t)n);              // alive, flag, side
   b += key_bytes(n);                        // first contraction pass: keys
   b += align16(4 * (size_t)((d + 31) / 32 + 1));  // contraction marks, one bit per entry
+  b += align16(sizeof(IT) * (size_t)n);     // row lengths
   b += align16(sizeof(IT) * (size_t)d);     // local adjacency
   return b + 64;
 }
@@ -80,8 +83,10 @@ struct Mem {
   uint8_t *alive, *flag, *side;
   uint32_t *kw;        // first contraction pass: 16-bit keys, two to a word
   uint32_t *ebits;     // one bit per local adjacency entry
+  IT *len;             // row i: adj[off[i] .. off[i] + len[i]), in any order
   IT *adj;
   size_t smem_used;    // bytes of dynamic shared memory the item occupies
+  __device__ __forceinline__ int end(int i) const { return off[i] + (int)len[i]; }
   bool off_in_smem;    // a global-slab item keeps its row offsets in shared memory
 };
 
@@ -106,6 +111,7 @@ __device__ __forceinline__ Mem<IT> carve(char *base, int n, int64_t d) {
   m.side = (uint8_t *)take((size_t)n);
   m.kw = (uint32_t *)take(key_bytes(n));
   m.ebits = (uint32_t *)take(4 * (size_t)((d + 31) / 32 + 1));
+  m.len = (IT *)take(sizeof(IT) * (size_t)n);
   m.adj = (IT *)take(sizeof(IT) * (size_t)d);
   m.smem_used = 0;
   m.off_in_smem = false;
@@ -313,7 +319,7 @@ __device__ __forceinline__ int components(const Mem<IT> &m, int n, Sh &sh, int32
     int changed = 0;
     for (int i = threadIdx.x; i < n; i += RB) {
       if (!m.alive[i]) continue;
-      const int b = m.off[i], e = m.off[i + 1];
+      const int b = m.off[i], e = m.end(i);
       if (e - b > 32) continue;
       for (int q = b; q < e; ++q) {
         const int j = m.adj[q];
@@ -330,7 +336,7 @@ __device__ __forceinline__ int components(const Mem<IT> &m, int n, Sh &sh, int32
       }
     }
     for (int i = warp; i < n; i += RW) {
-      const int b = m.off[i], e = m.off[i + 1];
+      const int b = m.off[i], e = m.end(i);
       if (!m.alive[i] || e - b <= 32) continue;
       for (int q = b + lane; q < e; q += 32) {
         const int j = m.adj[q];
@@ -392,7 +398,7 @@ __device__ __forceinline__ void afforest(const Mem<IT> &m, int n, int32_t *uf, i
   for (int r = 0; r < 2; ++r) {
     for (int i = threadIdx.x; i < n; i += RB) {
       if (!m.alive[i]) continue;
-      const int e = m.off[i + 1];
+      const int e = m.end(i);
       int q = cur[i];
       for (; q < e; ++q) {
         const int j = m.adj[q];
@@ -415,7 +421,7 @@ __device__ __forceinline__ void afforest(const Mem<IT> &m, int n, int32_t *uf, i
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int i = threadIdx.x; i < n; i += RB) {
     if (!m.alive[i]) continue;
-    const int e = m.off[i + 1];
+    const int e = m.end(i);
     if (e - cur[i] > 64 || uf_find(uf, i) == giant) continue;
     for (int q = cur[i]; q < e; ++q) {
       const int j = m.adj[q];
@@ -424,7 +430,7 @@ __device__ __forceinline__ void afforest(const Mem<IT> &m, int n, int32_t *uf, i
   }
   for (int i = warp; i < n; i += RW) {
     if (!m.alive[i]) continue;
-    const int e = m.off[i + 1];
+    const int e = m.end(i);
     if (e - cur[i] <= 64 || uf_find(uf, i) == giant) continue;
     for (int q = cur[i] + lane; q < e; q += 32) {
       const int j = m.adj[q];
@@ -667,7 +673,7 @@ __device__ __forceinline__ void scan_super_vertex(const Mem<IT> &m, const int32_
   const int mb = m.C[X], me = m.C[X + 1];
   if (me - mb == 1) {
     const int i = m.D[mb];
-    for (int e = m.off[i] + lane; e < m.off[i + 1]; e += 32) {
+    for (int e = m.off[i] + lane; e < m.end(i); e += 32) {
       const int j = m.adj[e];
       if (!m.alive[j]) continue;
       const int Y = grp[j];
@@ -677,7 +683,7 @@ __device__ __forceinline__ void scan_super_vertex(const Mem<IT> &m, const int32_
   } else {
     for (int q = mb + lane; q < me; q += 32) {
       const int i = m.D[q];
-      for (int e = m.off[i]; e < m.off[i + 1]; ++e) {
+      for (int e = m.off[i]; e < m.end(i); ++e) {
         const int j = m.adj[e];
         if (!m.alive[j]) continue;
         const int Y = grp[j];
@@ -879,7 +885,7 @@ __device__ __forceinline__ int first_pass(const Mem<IT> &m, int32_t *rep, int n,
           const int i = i0 + threadIdx.x;
           bool take = false;
           if (i < n && kh[i] < kcap) {
-            const int b = m.off[i], e = m.off[i + 1];
+            const int b = m.off[i], e = m.end(i);
             if (e - b > PULL_ROW) {
               lr[atomicAdd(&sh.ntouched, 1)] = i;
             } else {
@@ -901,7 +907,7 @@ __device__ __forceinline__ int first_pass(const Mem<IT> &m, int32_t *rep, int n,
         __syncthreads();
         const int nl = sh.ntouched;
         for (int k = warp; k < nl; k += RW) {
-          const int i = lr[k], b = m.off[i], e = m.off[i + 1];
+          const int i = lr[k], b = m.off[i], e = m.end(i);
           int c = 0;
           for (int q = b; q < e && c < kcap; q += 32) {
             const bool in = q + lane < e && (kh[(int)m.adj[q + lane]] & KEY_IN);
@@ -927,7 +933,7 @@ __device__ __forceinline__ int first_pass(const Mem<IT> &m, int32_t *rep, int n,
           if (lane < cnt) {
             const int v = queue[c0 + lane];
             b = m.off[v];
-            e = m.off[v + 1];
+            e = m.end(v);
           }
           for (int t = 0; t < cnt; t += 2) {
             const int src = t + (lane >> 4);  // at most 32, with cnt odd: the bounds are empty then
@@ -1033,7 +1039,7 @@ __device__ __forceinline__ int class_pass(const Mem<IT> &m, int32_t *rep, int n,
       const int rn = r == 2 ? 0 : r + 1;
       if (threadIdx.x == 0) sh.qn[rn] = 0;
       auto scan_row = [&](int i) {  // one member's row, by a warp
-        const int b = m.off[i], e = m.off[i + 1];
+        const int b = m.off[i], e = m.end(i);
         for (int q0 = b; q0 < e; q0 += 32) {
           bool take = false;
           int Y = -1;
@@ -1124,12 +1130,12 @@ __device__ __forceinline__ void ma_ordering_block(const Mem<IT> &m, const int32_
       // few members: a warp per member, lanes along its row
       for (int q = mb + warp; q < me; q += RW) {
         const int i = m.D[q];
-        for (int e = m.off[i] + lane; e < m.off[i + 1]; e += 32) visit(e);
+        for (int e = m.off[i] + lane; e < m.end(i); e += 32) visit(e);
       }
     } else {
       for (int q = mb + threadIdx.x; q < me; q += RB) {
         const int i = m.D[q];
-        for (int e = m.off[i]; e < m.off[i + 1]; ++e) visit(e);
+        for (int e = m.off[i]; e < m.end(i); ++e) visit(e);
       }
     }
     __syncthreads();
@@ -1488,7 +1494,7 @@ __device__ __forceinline__ void rows_pass(const Mem<IT> &m, int n, const int32_t
                                           Sel sel, F f) {
   for (int a = threadIdx.x; a < n; a += RB) {
     if (!m.alive[a]) continue;
-    const int b0 = m.off[a], e0 = m.off[a + 1];
+    const int b0 = m.off[a], e0 = m.end(a);
     if (e0 - b0 > FOREST_LONG_ROW || !sel(a)) continue;
     for (int q = b0; q < e0; ++q) f(a, q, (int)m.adj[q]);
   }
@@ -1496,7 +1502,7 @@ __device__ __forceinline__ void rows_pass(const Mem<IT> &m, int n, const int32_t
   for (int k = warp; k < nlr; k += RW) {
     const int a = lr[k];
     if (!sel(a)) continue;
-    for (int q = m.off[a] + lane; q < m.off[a + 1]; q += 32) f(a, q, (int)m.adj[q]);
+    for (int q = m.off[a] + lane; q < m.end(a); q += 32) f(a, q, (int)m.adj[q]);
   }
 }
 
@@ -1514,12 +1520,12 @@ __device__ __forceinline__ int forest_accept(const Mem<IT> &m, int n, int kcap, 
   int32_t *lr = m.D, *rep = m.G, *deg = m.H;
   uint32_t *used = m.ebits;
   volatile uint32_t *vu = used;
-  const int E = m.off[n];
+  const int E = m.off[n];  // entries the rows have room for
   if (threadIdx.x == 0) sh.ntouched = 0;
   __syncthreads();
   for (int i = threadIdx.x; i < n; i += RB) {
     rep[i] = m.alive[i] ? i : -1;
-    if (m.alive[i] && m.off[i + 1] - m.off[i] > FOREST_LONG_ROW) lr[atomicAdd(&sh.ntouched, 1)] = i;
+    if (m.alive[i] && (int)m.len[i] > FOREST_LONG_ROW) lr[atomicAdd(&sh.ntouched, 1)] = i;
   }
   __syncthreads();
   const int nlr = sh.ntouched;
@@ -2028,129 +2034,124 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
     carve_hot(m, n, P.smem_bytes);
   }
 
-  // global row start and degree of every member
+  // global row start and degree of every member; a local row gets room for
+  // all of its vertex's entries
   int64_t *gbeg = m.wide;
-  int32_t *pdeg = m.C, *cnt = m.D;
+  int32_t *deg0 = m.C, *cnt = m.D, *lr = m.G;
   for (int i = threadIdx.x; i < n; i += RB) {
     const int32_t v = __ldcg(&R.pool[vbeg + i]);
     m.gid[i] = v;
     const int64_t b = R.off[v];
+    const int32_t d = (int32_t)(R.off[v + 1] - b);
     gbeg[i] = b;
-    pdeg[i] = (int32_t)(R.off[v + 1] - b);
-    cnt[i] = 0;
+    deg0[i] = d;
+    m.off[i] = d;
+    if (d > LONG_ROW) cnt[i] = 0;
+    m.alive[i] = 1;
   }
+  if (threadIdx.x == 0) sh.ntouched = 0;
   __syncthreads();
-  const int D = block_scan_array(pdeg, n, sh);
-  if (threadIdx.x == 0) pdeg[n] = D;
+  const int D = block_scan_array(m.off, n, sh);
+  if (threadIdx.x == 0) m.off[n] = D;
   __syncthreads();
   prof_stamp(P, sh, 1);
 
-  // 1. extraction, flat over all D adjacency entries of the members so that
-  // every thread keeps independent loads in flight: entry f of row i keeps
-  // its neighbour u iff slot[u] names this item; tmp[f] = local id or ~0
-  IT *tmp = m.adj;
-  const IT NONE = (IT)~(IT)0;
-  if (!SM) {
-    // items in the global slab: their row bounds are global too, so a
-    // per-entry row cursor would put a dependent global load on every
-    // entry; instead each warp takes two rows at a time, reads their bounds
-    // once, and its lanes walk the rows together (64 neighbour loads and 64
-    // slot gathers in flight per warp)
-    for (int r0 = 2 * warp; r0 < n; r0 += 2 * RW) {
-      const int r1 = r0 + 1 < n ? r0 + 1 : r0;
-      const int o0 = pdeg[r0], d0 = pdeg[r0 + 1] - o0;
-      const int o1 = pdeg[r1], d1 = r1 != r0 ? pdeg[r1 + 1] - o1 : 0;
-      const int64_t g0 = gbeg[r0], g1 = gbeg[r1];
-      int c0 = 0, c1 = 0;
-      const int dm = d0 > d1 ? d0 : d1;
-      for (int k = lane; k - lane < dm; k += 32) {
-        const bool a0 = k < d0, a1 = k < d1;
-        const int32_t u0 = a0 ? R.adj[g0 + k] : 0;
-        const int32_t u1 = a1 ? R.adj[g1 + k] : 0;
-        const unsigned long long s0 = a0 ? __ldcg(&R.slot[u0]) : 0ull;
-        const unsigned long long s1 = a1 ? __ldcg(&R.slot[u1]) : 0ull;
-        const bool h0 = a0 && (unsigned)(s0 >> 32) == queue_tag(seq);
-        const bool h1 = a1 && (unsigned)(s1 >> 32) == queue_tag(seq);
-        if (a0) tmp[o0 + k] = h0 ? (IT)(unsigned)(s0 & 0xffffffffu) : NONE;
-        if (a1) tmp[o1 + k] = h1 ? (IT)(unsigned)(s1 & 0xffffffffu) : NONE;
-        c0 += __popc(__ballot_sync(FULL, h0));
-        c1 += __popc(__ballot_sync(FULL, h1));
-      }
-      if (lane == 0) {
-        cnt[r0] = c0;
-        if (r1 != r0) cnt[r1] = c1;
-      }
-    }
-  } else {
-    // warp w owns entries [w*chunk, (w+1)*chunk); lane l takes every 32nd
-    // entry of it, four at a time, following its row with a cursor
-    const int chunk = (D + RW - 1) / RW;
-    const int f0 = warp * chunk, f1 = min(D, f0 + chunk);
-    int row = 0;
-    if (f0 + lane < f1) {
-      int lo = 0, hi = n;  // largest i with pdeg[i] <= f0 + lane
-      while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (pdeg[mid] <= f0 + lane) lo = mid; else hi = mid;
-      }
-      row = lo;
-    }
-    for (int fb = f0 + lane; fb < f1; fb += 128) {
-      int fs[4], rs[4];
-      int32_t us[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int f = fb + 32 * k;
-        fs[k] = f;
-        if (f < f1) {
-          while (pdeg[row + 1] <= f) ++row;
-          rs[k] = row;
-          us[k] = R.adj[gbeg[row] + (f - pdeg[row])];
+  // 1. extraction: entry (i, u) stays iff slot[u] names this item, as u's
+  // local id; the entries of a local row are in any order.  What bounds it is
+  // the latency of two dependent gathers an entry (neighbour, then its slot),
+  // so every lane keeps four entries in flight whatever the row lengths: a
+  // warp takes up to 32 rows, lane r holding row r's bounds, and walks their
+  // entries as one flat range, 128 at a time; an entry's row is found by a
+  // binary search over the lanes' degree prefix, its place by a ballot and
+  // the count of hits that the row's lane holds.  Long rows are shared by
+  // all warps in segments of 128 entries.  A cluster of 47,000 vertices and
+  // 2.15M entries takes 9.3M cycles (two rows a warp at a time, all entries
+  // kept and compacted by a second pass: 20.7M; eight rows a warp, each lane
+  // waiting for the longest: 13.4M).
+  {
+    const uint32_t tag = queue_tag(seq);
+    const unsigned lt = lanemask_lt();
+    const int per = min(32, (n + RW - 1) / RW);
+    for (int r0 = warp * per; r0 < n; r0 += RW * per) {
+      const int rows = min(per, n - r0);
+      int o = 0, d = 0;
+      long long g = 0;
+      bool is_long = false;
+      if (lane < rows) {
+        const int i = r0 + lane;
+        o = m.off[i];
+        d = deg0[i];
+        g = gbeg[i];
+        is_long = d > LONG_ROW;
+        if (is_long) {
+          lr[atomicAdd(&sh.ntouched, 1)] = i;
+          d = 0;
         }
       }
-      unsigned long long sl[4];
+      const int inc = warp_inclusive_scan(d), exc = inc - d;
+      const int total = __shfl_sync(FULL, inc, 31);
+      g -= exc;
+      int c = 0;  // hits of the lane's row so far
+      for (int f0 = 0; f0 < total; f0 += 128) {
+        int row[4];
+        int32_t u[4];
+        unsigned long long sl[4];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) sl[k] = fs[k] < f1 ? __ldcg(&R.slot[us[k]]) : 0ull;
+        for (int z = 0; z < 4; ++z) {
+          const int f = f0 + 32 * z + lane;
+          int lo = 0;  // rows that end at or before f
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        if (fs[k] >= f1) continue;
-        const bool hit = (unsigned)(sl[k] >> 32) == queue_tag(seq);
-        tmp[fs[k]] = hit ? (IT)(unsigned)(sl[k] & 0xffffffffu) : NONE;
-        if (hit) atomicAdd(&cnt[rs[k]], 1);
+          for (int st = 16; st > 0; st >>= 1)
+            if (__shfl_sync(FULL, inc, lo + st - 1) <= f) lo += st;
+          row[z] = lo;
+          const long long gr = __shfl_sync(FULL, g, lo);
+          u[z] = f < total ? R.adj[gr + f] : -1;
+        }
+#pragma unroll
+        for (int z = 0; z < 4; ++z) sl[z] = u[z] >= 0 ? __ldcg(&R.slot[u[z]]) : ~0ull;
+#pragma unroll
+        for (int z = 0; z < 4; ++z) {
+          const bool hit = (uint32_t)(sl[z] >> 32) == tag;
+          const unsigned b = __ballot_sync(FULL, hit);
+          // the lane's row within these 32 entries
+          const int base = f0 + 32 * z;
+          const int lo = min(max(exc - base, 0), 32), hi = min(max(inc - base, 0), 32);
+          const unsigned mine = (unsigned)((1ull << hi) - (1ull << lo));
+          const unsigned rm = __shfl_sync(FULL, mine, row[z]);
+          const int at = __shfl_sync(FULL, o + c, row[z]);
+          if (hit) m.adj[at + __popc(b & rm & lt)] = (IT)(unsigned)(sl[z] & 0xffffffffu);
+          c += __popc(b & mine);
+        }
+      }
+      if (lane < rows && !is_long) m.len[r0 + lane] = (IT)c;
+    }
+    __syncthreads();
+    const int nl = sh.ntouched;
+    for (int k = 0; k < nl; ++k) {
+      const int i = lr[k], d = deg0[i], o = m.off[i];
+      const int64_t g = gbeg[i];
+      for (int f0 = 128 * ((warp + k) % RW); f0 < d; f0 += 128 * RW) {
+        int32_t u[4];
+        unsigned long long sl[4];
+#pragma unroll
+        for (int z = 0; z < 4; ++z) u[z] = f0 + 32 * z + lane < d ? R.adj[g + f0 + 32 * z + lane] : -1;
+#pragma unroll
+        for (int z = 0; z < 4; ++z) sl[z] = u[z] >= 0 ? __ldcg(&R.slot[u[z]]) : ~0ull;
+#pragma unroll
+        for (int z = 0; z < 4; ++z) {
+          const bool hit = (uint32_t)(sl[z] >> 32) == tag;
+          const unsigned b = __ballot_sync(FULL, hit);
+          int at = 0;
+          if (lane == 0 && b) at = atomicAdd(&cnt[i], __popc(b));
+          at = __shfl_sync(FULL, at, 0);
+          if (hit) m.adj[o + at + __popc(b & lanemask_lt())] = (IT)(unsigned)(sl[z] & 0xffffffffu);
+        }
       }
     }
+    __syncthreads();
+    for (int k = threadIdx.x; k < nl; k += RB) m.len[lr[k]] = (IT)cnt[lr[k]];
+    if (threadIdx.x == 0) sh.ntouched = 0;
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < n; i += RB) m.off[i] = cnt[i];
-  __syncthreads();
-  const int E = block_scan_array(m.off, n, sh);
-  if (threadIdx.x == 0) m.off[n] = E;
-  // order-preserving compaction of tmp into the local adjacency, in chunks
-  // read fully into registers before any write (destinations never pass the
-  // chunk's own sources)
-  {
-    constexpr int CI = 4;
-    int carry = 0;
-    for (int c0 = 0; c0 < D; c0 += RB * CI) {
-      IT v[CI];
-      int k = 0;
-#pragma unroll
-      for (int q = 0; q < CI; ++q) {
-        const int f = c0 + threadIdx.x * CI + q;
-        v[q] = f < D ? tmp[f] : NONE;
-        k += v[q] != NONE;
-      }
-      int tot;
-      int ex = block_exclusive_scan<RB>(k, &tot, sh.scan);
-      int w = carry + ex;
-#pragma unroll
-      for (int q = 0; q < CI; ++q)
-        if (v[q] != NONE) m.adj[w++] = v[q];
-      carry += tot;
-      __syncthreads();
-    }
-  }
-  for (int i = threadIdx.x; i < n; i += RB) m.alive[i] = 1;
   __syncthreads();
   if (threadIdx.x == 0) {
     add_ll(&ctr->items, 1ll);
@@ -2159,7 +2160,7 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
     // and its label (4 + 4 B); re-inducing a part after a split reads the
     // entries again (8 B each)
     add_ll(&ctr->alg_bytes, (long long)((it.flags & ITEM_TOP) ? 8 * n : 0) + 8 * (long long)D);
-    sh.pf_E = E;
+    sh.pf_E = D;
   }
   prof_stamp(P, sh, 2);
 
@@ -2187,7 +2188,7 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
 
   // 3. peel (round-synchronous, T recomputed from the alive count)
   int32_t *deg = m.A;
-  for (int i = threadIdx.x; i < n; i += RB) deg[i] = m.off[i + 1] - m.off[i];
+  for (int i = threadIdx.x; i < n; i += RB) deg[i] = (int32_t)m.len[i];
   __syncthreads();
   const int n_item = nalive;
   for (;;) {
@@ -2202,7 +2203,7 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
     if (rem == 0) break;
     for (int i = warp; i < n; i += RW) {
       if (!m.flag[i]) continue;
-      for (int e = m.off[i] + lane; e < m.off[i + 1]; e += 32) atomicSub(&deg[m.adj[e]], 1);
+      for (int e = m.off[i] + lane; e < m.end(i); e += 32) atomicSub(&deg[m.adj[e]], 1);
       if (lane == 0) m.alive[i] = 0;
     }
     __syncthreads();
@@ -2378,7 +2379,7 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
       };
       for (int a = threadIdx.x; a < n; a += RB) {
         if (!m.alive[a] || rep[a] == big) continue;
-        const int b0 = m.off[a], e0 = m.off[a + 1];
+        const int b0 = m.off[a], e0 = m.end(a);
         if (e0 - b0 > 32) {
           lr[atomicAdd(&sh.ntouched, 1)] = a;
           continue;
@@ -2391,7 +2392,7 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
         const int nl = sh.ntouched;
         for (int k = warp; k < nl; k += RW) {
           const int a = lr[k], A = idx[rep[a]];
-          for (int q = m.off[a] + lane; q < m.off[a + 1]; q += 32) weigh(A, (int)m.adj[q]);
+          for (int q = m.off[a] + lane; q < m.end(a); q += 32) weigh(A, (int)m.adj[q]);
         }
       }
       __syncthreads();
@@ -2509,9 +2510,11 @@ __device__ int run_item(const RefineParams &P, unsigned long long seq, const Ite
     dsum += R.off[v + 1] - R.off[v];
   }
   dsum = block_sum_ll(dsum, sh);
+  // at 65,535 vertices the working memory is far above what a CTA can hold
+  // in shared memory: 32-bit local ids only occur in the slab
   const bool narrow = n < 65535;
   const size_t need = narrow ? ws_bytes<uint16_t>(n, dsum) : ws_bytes<int32_t>(n, dsum);
-  const bool in_smem = need <= P.smem_bytes;
+  const bool in_smem = narrow && need <= P.smem_bytes;
   if (!in_smem && (need > P.slab_bytes || dsum >= (1ll << 31))) {
     if (threadIdx.x == 0) {
       atomicOr(&P.ctr->error, DERR_CAPACITY);
@@ -2520,9 +2523,7 @@ __device__ int run_item(const RefineParams &P, unsigned long long seq, const Ite
     return OUT_ERROR;
   }
   if (threadIdx.x == 0) sh.used_slab = !in_smem;
-  if (in_smem)
-    return narrow ? process_item<uint16_t, true>(P, seq, it, slab, dsum, sh)
-                  : process_item<int32_t, true>(P, seq, it, slab, dsum, sh);
+  if (in_smem) return process_item<uint16_t, true>(P, seq, it, slab, dsum, sh);
   return narrow ? process_item<uint16_t, false>(P, seq, it, slab, dsum, sh)
                 : process_item<int32_t, false>(P, seq, it, slab, dsum, sh);
 }
