@@ -772,11 +772,54 @@ __device__ __forceinline__ void ma_ordering(const Mem<IT> &m, const int32_t *grp
 constexpr unsigned KEY_IN = 0x8000u;    // added, or queued to be
 constexpr unsigned KEY_DEAD = 0x4000u;  // peeled: never below kcap, never added
 constexpr int KEY_MAX = 0x3fff;         // largest kcap the 16-bit keys hold
-// A round looks from the unadded vertices' side once the vertices added in
-// the round before outnumber a quarter of them: their rows stop at kcap
-// added neighbours, and the last rounds add most of the vertices at once.
+// A round looks from the unadded vertices' side when the vertices added in
+// the round before are at least twice as many: the last rounds add most of
+// the vertices at once, and an unadded one stops at kcap added neighbours,
+// most often within its first 32 entries.
 constexpr int PULL_MIN = 64;
-constexpr int PULL_ROW = 96;  // longer rows are looked through by a warp
+constexpr int PULL_STEP = 32;
+
+// The entries of up to 32 rows, lane r holding row r = adj[b .. b + d), walked
+// by one warp as one flat range.  Calls fn(j, base) for every 128 entries:
+// j[z] the lane's entry base + 32 z + lane (-1: none); the lane's own row is
+// the range [exc, exc + d) of them.  Every lane calls.
+template <typename IT, typename Fn>
+__device__ __forceinline__ void flat_rows(const IT *adj, int b, int d, int &exc, Fn fn) {
+  const int lane = threadIdx.x & 31;
+  const int inc = warp_inclusive_scan(d);
+  exc = inc - d;
+  const int total = __shfl_sync(FULL, inc, 31), g = b - exc;
+  for (int f0 = 0; f0 < total; f0 += 128) {
+    int j[4], lo[4] = {0, 0, 0, 0};  // lo: rows that end at or before the entry
+#pragma unroll
+    for (int st = 16; st > 0; st >>= 1)
+#pragma unroll
+      for (int z = 0; z < 4; ++z)
+        if (__shfl_sync(FULL, inc, lo[z] + st - 1) <= f0 + 32 * z + lane) lo[z] += st;
+#pragma unroll
+    for (int z = 0; z < 4; ++z) {
+      const int f = f0 + 32 * z + lane;
+      const int gr = __shfl_sync(FULL, g, lo[z]);
+      j[z] = f < total ? (int)adj[gr + f] : -1;
+    }
+    fn(j, f0);
+  }
+}
+
+// The same for a single row adj[b .. b + d).
+template <typename IT, typename Fn>
+__device__ __forceinline__ void one_row(const IT *adj, int b, int d, Fn fn) {
+  const int lane = threadIdx.x & 31;
+  for (int f0 = 0; f0 < d; f0 += 128) {
+    int j[4];
+#pragma unroll
+    for (int z = 0; z < 4; ++z) {
+      const int f = f0 + 32 * z + lane;
+      j[z] = f < d ? (int)adj[b + f] : -1;
+    }
+    fn(j, f0);
+  }
+}
 
 // Block maximum of a 32- or 64-bit value; every thread returns it.  Two
 // calls need a barrier between them.
@@ -806,6 +849,27 @@ __device__ __forceinline__ int warp_push(bool take, int32_t v, int32_t *queue, i
   at = __shfl_sync(FULL, at, leader);
   if (take) queue[base + at + __popc(b & lanemask_lt())] = v;
   return __popc(b);
+}
+
+// The same for up to four vertices a lane, with one atomic.
+__device__ __forceinline__ void warp_push4(const bool (&take)[4], const int (&v)[4],
+                                           int32_t *queue, int base, int32_t *cnt) {
+  unsigned b[4];
+  int k = 0;
+#pragma unroll
+  for (int z = 0; z < 4; ++z) {
+    b[z] = __ballot_sync(FULL, take[z]);
+    k += __popc(b[z]);
+  }
+  if (k == 0) return;
+  int at = 0;
+  if ((threadIdx.x & 31) == 0) at = atomicAdd(cnt, k);
+  at = base + __shfl_sync(FULL, at, 0);
+#pragma unroll
+  for (int z = 0; z < 4; ++z) {
+    if (take[z]) queue[at + __popc(b[z] & lanemask_lt())] = v[z];
+    at += __popc(b[z]);
+  }
 }
 
 // The first contraction pass, on the item's own vertices (every super-vertex
@@ -870,99 +934,97 @@ __device__ __forceinline__ int first_pass(const Mem<IT> &m, int32_t *rep, int n,
       kh[X] = (uint16_t)KEY_IN;
     }
     int head = tail++;
-    bool pull = false;
     __syncthreads();
     while (head < tail && tail < nalive) {
-      const int F = tail - head;
+      const int F = tail - head, U = nalive - tail;
       int32_t *qn = &sh.qn[r];
       const int rn = r == 2 ? 0 : r + 1;
       if (threadIdx.x == 0) sh.qn[rn] = 0;
-      pull = pull || (F >= PULL_MIN && 4 * F >= nalive - tail);
-      if (pull) {
-        // every unadded vertex counts its added neighbours afresh (a round
-        // that adds none leaves exact keys)
+      if (F >= PULL_MIN && F >= 2 * U) {
+        // every unadded vertex counts its added neighbours afresh; those it
+        // takes are marked only after the round, so that the keys of the
+        // rest are exact
         for (int i0 = 0; i0 < n; i0 += RB) {
           const int i = i0 + threadIdx.x;
-          bool take = false;
-          if (i < n && kh[i] < kcap) {
-            const int b = m.off[i], e = m.end(i);
-            if (e - b > PULL_ROW) {
-              lr[atomicAdd(&sh.ntouched, 1)] = i;
-            } else {
-              int c = 0;
-              for (int q = b; q < e && c < kcap; q += 4) {
-                int j[4];
+          warp_push(i < n && kh[i] < kcap, i, lr, 0, &sh.ntouched);
+        }
+        __syncthreads();
+        const int nl = sh.ntouched;
+        const int per = min(32, (nl + RW - 1) / RW);
+        for (int c0 = warp * per; c0 < nl; c0 += RW * per) {
+          int i = -1, b = 0, left = 0, c = 0;
+          if (lane < min(per, nl - c0)) {
+            i = lr[c0 + lane];
+            b = m.off[i];
+            left = (int)m.len[i];
+          }
+          for (int st = PULL_STEP; __any_sync(FULL, left > 0); st *= 2) {
+            const int d = min(left, st);
+            int exc;
+            flat_rows(m.adj, b, d, exc, [&](const int (&j)[4], int f0) {
+              unsigned k[4];
 #pragma unroll
-                for (int z = 0; z < 4; ++z) j[z] = (int)m.adj[q + z < e ? q + z : q];
+              for (int z = 0; z < 4; ++z) k[z] = j[z] >= 0 ? kh[j[z]] : 0u;
 #pragma unroll
-                for (int z = 0; z < 4; ++z) c += (q + z < e && (kh[j[z]] & KEY_IN)) ? 1 : 0;
+              for (int z = 0; z < 4; ++z) {
+                // hits within the lane's row
+                const int lo = min(max(exc - f0 - 32 * z, 0), 32);
+                const int hi = min(max(exc + d - f0 - 32 * z, 0), 32);
+                const unsigned mine = (unsigned)((1ull << hi) - (1ull << lo));
+                c += __popc(__ballot_sync(FULL, (k[z] & KEY_IN) != 0u) & mine);
               }
-              take = c >= kcap;
-              kh[i] = (uint16_t)(take ? KEY_IN : (unsigned)c);
-              if (take) rep[i] = phases;
-            }
+            });
+            b += d;
+            left = c >= kcap ? 0 : left - d;
+          }
+          const bool take = c >= kcap;
+          if (i >= 0) {
+            kh[i] = (uint16_t)(take ? KEY_DEAD : (unsigned)c);
+            if (take) rep[i] = phases;
           }
           warp_push(take, i, queue, tail, qn);
         }
         __syncthreads();
-        const int nl = sh.ntouched;
-        for (int k = warp; k < nl; k += RW) {
-          const int i = lr[k], b = m.off[i], e = m.end(i);
-          int c = 0;
-          for (int q = b; q < e && c < kcap; q += 32) {
-            const bool in = q + lane < e && (kh[(int)m.adj[q + lane]] & KEY_IN);
-            c += __popc(__ballot_sync(FULL, in));
-          }
-          const bool take = c >= kcap;
-          if (lane == 0) {
-            kh[i] = (uint16_t)(take ? KEY_IN : (unsigned)c);
-            if (take) rep[i] = phases;
-          }
-          warp_push(take && lane == 0, i, queue, tail, qn);
-        }
-        __syncthreads();
+        for (int q = threadIdx.x; q < *(volatile int32_t *)qn; q += RB)
+          kh[queue[tail + q]] = (uint16_t)KEY_IN;
         if (threadIdx.x == 0) sh.ntouched = 0;
       } else {
-        // the vertices added last raise their neighbours' keys: a warp takes
-        // up to 32 of them, reads their row bounds at once and walks two
-        // rows at a time, 64 entries of each in flight
-        const int per = min(32, (F + RW - 1) / RW);
-        for (int c0 = head + warp * per; c0 < tail; c0 += RW * per) {
-          const int cnt = min(per, tail - c0);
-          int b = 0, e = 0;
-          if (lane < cnt) {
-            const int v = queue[c0 + lane];
-            b = m.off[v];
-            e = m.end(v);
-          }
-          for (int t = 0; t < cnt; t += 2) {
-            const int src = t + (lane >> 4);  // at most 32, with cnt odd: the bounds are empty then
-            const int bb = __shfl_sync(FULL, b, src & 31), ee0 = __shfl_sync(FULL, e, src & 31);
-            const int ee = src < cnt ? ee0 : bb;
-            const int len = max(ee - bb, __shfl_xor_sync(FULL, ee - bb, 16));
-            for (int q0 = 0; q0 < len; q0 += 64) {
-              int j[4];
+        // the vertices added last raise their neighbours' keys; loads and
+        // atomics of four entries a lane overlap
+        auto raise = [&](const int (&j)[4], int) {
+          unsigned k[4], old[4];
+          bool take[4];
 #pragma unroll
-              for (int z = 0; z < 4; ++z) {
-                const int q = bb + q0 + 16 * z + (lane & 15);
-                j[z] = q < ee ? (int)m.adj[q] : -1;
-              }
+          for (int z = 0; z < 4; ++z) k[z] = j[z] >= 0 ? kh[j[z]] : KEY_DEAD;
 #pragma unroll
-              for (int z = 0; z < 4; ++z) {
-                if (q0 + 16 * z >= len) break;
-                bool take = false;
-                if (j[z] >= 0 && kh[j[z]] < kcap) {
-                  const int sft = (j[z] & 1) * 16;
-                  const unsigned old = atomicAdd(&kw[j[z] >> 1], 1u << sft);
-                  take = (int)((old >> sft) & 0xffffu) + 1 == kcap;
-                  if (take) {
-                    atomicOr(&kw[j[z] >> 1], KEY_IN << sft);
-                    rep[j[z]] = phases;
-                  }
-                }
-                warp_push(take, j[z], queue, tail, qn);
-              }
+          for (int z = 0; z < 4; ++z)
+            old[z] = k[z] < (unsigned)kcap ? atomicAdd(&kw[j[z] >> 1], 1u << ((j[z] & 1) * 16)) : 0u;
+#pragma unroll
+          for (int z = 0; z < 4; ++z) {
+            take[z] = k[z] < (unsigned)kcap &&
+                      ((old[z] >> ((j[z] & 1) * 16)) & 0xffffu) + 1u == (unsigned)kcap;
+            if (take[z]) {
+              atomicOr(&kw[j[z] >> 1], KEY_IN << ((j[z] & 1) * 16));
+              rep[j[z]] = phases;
             }
+          }
+          warp_push4(take, j, queue, tail, qn);
+        };
+        if (F <= RW) {
+          if (warp < F) {
+            const int v = queue[head + warp];
+            one_row(m.adj, m.off[v], (int)m.len[v], raise);
+          }
+        } else {
+          const int per = min(32, (F + RW - 1) / RW);
+          for (int c0 = head + warp * per; c0 < tail; c0 += RW * per) {
+            int b = 0, d = 0, exc;
+            if (lane < min(per, tail - c0)) {
+              const int v = queue[c0 + lane];
+              b = m.off[v];
+              d = (int)m.len[v];
+            }
+            flat_rows(m.adj, b, d, exc, raise);
           }
         }
       }
@@ -1185,7 +1247,7 @@ __device__ __forceinline__ void dense_fold(int32_t *w, int nsv, int r, int l) {
 __device__ __forceinline__ void dense_order(const int32_t *w, int nsv, uint32_t live, int kcap,
                                             int32_t *duf, int &s, int &t, int &cut, bool &merged) {
   const int l = threadIdx.x & 31;
-  long long key = 0;
+  unsigned key = 0;  // at most the item's edges, below 2^30
   bool added = !((live >> l) & 1u);
   const int cnt = __popc(live);
   s = t = -1;
@@ -1193,24 +1255,17 @@ __device__ __forceinline__ void dense_order(const int32_t *w, int nsv, uint32_t 
   merged = false;
   for (int step = 0; step < cnt; ++step) {
     // largest key, ties to the smallest index
-    const unsigned long long pk =
-        added ? 0ull : (((unsigned long long)key << 6) | (unsigned long long)(63 - l)) + 1ull;
-    unsigned long long best = pk;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long x = __shfl_xor_sync(FULL, best, o);
-      best = x > best ? x : best;
-    }
-    const int X = 63 - (int)((best - 1ull) & 63ull);
+    const unsigned top = __reduce_max_sync(FULL, added ? 0u : key);
+    const int X = __ffs(__ballot_sync(FULL, !added && key == top)) - 1;
     s = t;
     t = X;
-    cut = (int)((best - 1ull) >> 6);
+    cut = (int)top;
     added |= l == X;
     const int wx = l < nsv ? w[X * nsv + l] : 0;
     if (!added && wx > 0) {
-      long long nk = key + wx;
-      if (kcap > 0 && nk >= kcap) {
-        nk = kcap;
+      unsigned nk = key + (unsigned)wx;
+      if (kcap > 0 && nk >= (unsigned)kcap) {
+        nk = (unsigned)kcap;
         // merge l into X's set (duf links point to smaller indices)
         volatile int32_t *vd = duf;
         int a = X, b = l;
@@ -1339,7 +1394,7 @@ __device__ __forceinline__ void dense_order_w(const int32_t *w, int nsv, const u
                                               int kcap, int32_t *duf, int &s, int &t, int &cut,
                                               bool &merged) {
   const int l = threadIdx.x & 31;
-  long long key[K];
+  unsigned key[K];  // at most the item's edges, below 2^30
   bool added[K];
   int cnt = 0;
 #pragma unroll
@@ -1353,32 +1408,27 @@ __device__ __forceinline__ void dense_order_w(const int32_t *w, int nsv, const u
   merged = false;
   for (int step = 0; step < cnt; ++step) {
     // largest key, ties to the smallest index
-    unsigned long long best = 0ull;
+    unsigned best = 0u;
 #pragma unroll
-    for (int j = 0; j < K; ++j) {
-      const unsigned long long pk =
-          added[j] ? 0ull
-                   : (((unsigned long long)key[j] << 7) | (unsigned long long)(127 - (l + 32 * j))) + 1ull;
-      best = pk > best ? pk : best;
-    }
+    for (int j = 0; j < K; ++j) best = max(best, added[j] ? 0u : key[j]);
+    best = __reduce_max_sync(FULL, best);
+    unsigned first = 0xffffffffu;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long x = __shfl_xor_sync(FULL, best, o);
-      best = x > best ? x : best;
-    }
-    const int X = 127 - (int)((best - 1ull) & 127ull);
+    for (int j = K - 1; j >= 0; --j)
+      if (!added[j] && key[j] == best) first = (unsigned)(l + 32 * j);
+    const int X = (int)__reduce_min_sync(FULL, first);
     s = t;
     t = X;
-    cut = (int)((best - 1ull) >> 7);
+    cut = (int)best;
 #pragma unroll
     for (int j = 0; j < K; ++j) {
       const int idx = l + 32 * j;
       added[j] |= idx == X;
       const int wx = idx < nsv ? w[X * nsv + idx] : 0;
       if (!added[j] && wx > 0) {
-        long long nk = key[j] + wx;
-        if (kcap > 0 && nk >= kcap) {
-          nk = kcap;
+        unsigned nk = key[j] + (unsigned)wx;
+        if (kcap > 0 && nk >= (unsigned)kcap) {
+          nk = (unsigned)kcap;
           volatile int32_t *vd = duf;
           int a = X, b = idx;
           for (;;) {
@@ -2350,7 +2400,7 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
       // few super-vertices left: their weight matrix, then the dense finish.
       // Rows of the largest one (most often it holds nearly all vertices)
       // are not looked through: its weights come from the other ends.
-      int32_t *idx = m.C, *lr = m.D, *rank = m.H;
+      int32_t *idx = m.C, *lr = m.D, *roots = m.H;
       int32_t *w = wmat;
       if (threadIdx.x < 32) {  // the set of most of 32 spread vertices
         const int v = (int)(((long long)lane * n) / 32);
@@ -2360,13 +2410,21 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
             warp_max(r >= 0 ? ((unsigned long long)__popc(peers) << 32) | (unsigned)r : 0ull);
         if (lane == 0) sh.i0 = best ? (int)(best & 0xffffffffu) : -1;
       }
-      for (int i = threadIdx.x; i < n; i += RB) rank[i] = (m.alive[i] && rep[i] == i) ? 1 : 0;
-      for (int q = threadIdx.x; q < nsv * nsv; q += RB) w[q] = 0;
-      if (threadIdx.x == 0) sh.ntouched = 0;
+      if (threadIdx.x == 0) sh.ntouched = sh.qn[0] = 0;
       __syncthreads();
-      block_scan_array(rank, n, sh);
-      for (int i = threadIdx.x; i < n; i += RB)
-        if (m.alive[i] && rep[i] == i) idx[i] = rank[i];
+      // the sets' smallest members, each one's index the number of smaller ones
+      for (int i0 = 0; i0 < n; i0 += RB) {
+        const int i = i0 + threadIdx.x;
+        warp_push(i < n && rep[i] == i, i, roots, 0, &sh.qn[0]);
+      }
+      for (int q = threadIdx.x; q < nsv * nsv; q += RB) w[q] = 0;
+      __syncthreads();
+      for (int k = threadIdx.x; k < nsv; k += RB) {
+        const int r = roots[k];
+        int at = 0;
+        for (int q = 0; q < nsv; ++q) at += roots[q] < r;
+        idx[r] = at;
+      }
       __syncthreads();
       const int big = sh.i0;
       auto weigh = [&](int A, int u) {  // the entry from a member of A to u
