@@ -45,6 +45,9 @@ constexpr size_t SMEM_MAX_BYTES = 227 * 1024;  // opt-in limit per CTA
 // generic ones.
 extern __shared__ __align__(16) char wcc_dyn_smem[];
 
+// Components that a contraction pass finds one after the other; beyond that
+// many the union-find finds all at once.
+constexpr int MAX_COMP = 32;
 // Rows of more entries are extracted by all warps together.
 constexpr int LONG_ROW = 1024;
 // Most small input clusters a CTA claims at once (see k_refine).  With one per
@@ -296,87 +299,9 @@ __device__ long long block_sum_ll(long long v, Sh &sh) {
   return tot;
 }
 
-// ---- connected components of the alive vertices ----------------------------
-// Hook-and-shortcut rounds: every alive edge (i, j) lowers the label of the
-// larger of f[i], f[j] to the smaller one (atomicMin), then every label is
-// shortcut to its label's label until stable; rounds repeat until neither
-// step changes anything.  Labels only decrease and stay ids of the same
-// component, so the fixpoint labels each component with its smallest id.
-// f[i] = that id (-1 for dead vertices; f defaults to B); returns the number
-// of components.  With emask, only the adjacency entries whose bit is set
-// count as edges (an undirected edge may be marked on either of its two
-// entries).
-template <typename IT>
-__device__ __forceinline__ int components(const Mem<IT> &m, int n, Sh &sh, int32_t *f = nullptr,
-                          const uint32_t *emask = nullptr) {
-  if (f == nullptr) f = m.B;
-  volatile int32_t *vf = f;
-  for (int i = threadIdx.x; i < n; i += RB) f[i] = m.alive[i] ? i : -1;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int round = 0; round <= n; ++round) {
-    if (threadIdx.x == 0) sh.changed = 0;
-    __syncthreads();
-    int changed = 0;
-    for (int i = threadIdx.x; i < n; i += RB) {
-      if (!m.alive[i]) continue;
-      const int b = m.off[i], e = m.end(i);
-      if (e - b > 32) continue;
-      for (int q = b; q < e; ++q) {
-        const int j = m.adj[q];
-        if (emask) {
-          if (!(emask[q >> 5] & (1u << (q & 31)))) continue;
-        } else if (j <= i || !m.alive[j]) {
-          continue;
-        }
-        const int a = vf[i], c = vf[j];
-        if (a != c) {
-          const int hi = a > c ? a : c, lo = a > c ? c : a;
-          if (atomicMin(&f[hi], lo) > lo) changed = 1;
-        }
-      }
-    }
-    for (int i = warp; i < n; i += RW) {
-      const int b = m.off[i], e = m.end(i);
-      if (!m.alive[i] || e - b <= 32) continue;
-      for (int q = b + lane; q < e; q += 32) {
-        const int j = m.adj[q];
-        if (emask) {
-          if (!(emask[q >> 5] & (1u << (q & 31)))) continue;
-        } else if (j <= i || !m.alive[j]) {
-          continue;
-        }
-        const int a = vf[i], c = vf[j];
-        if (a != c) {
-          const int hi = a > c ? a : c, lo = a > c ? c : a;
-          if (atomicMin(&f[hi], lo) > lo) changed = 1;
-        }
-      }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < n; i += RB) {
-      if (!m.alive[i]) continue;
-      int x = vf[i];
-      int y = vf[x];
-      while (y != x) {
-        x = y;
-        y = vf[x];
-      }
-      if (vf[i] != x) {
-        vf[i] = x;
-        changed = 1;
-      }
-    }
-    if (changed) sh.changed = 1;
-    __syncthreads();
-    if (!sh.changed) break;
-  }
-  int roots = 0;
-  for (int i = threadIdx.x; i < n; i += RB) roots += (m.alive[i] && f[i] == i);
-  return block_sum_int(roots, sh);
-}
-
 // ---- connected components (Afforest-style) ---------------------------------
-// Union-find over the alive vertices (uf, root = smallest id): every vertex
+// For items of more than MAX_COMP components (fewer come out of a contraction
+// pass, see first_pass).  Union-find over the alive vertices (uf, root = smallest id): every vertex
 // first links along its first two alive neighbours, the sets are
 // compressed, and then only vertices outside the set of the smallest alive
 // vertex process the rest of their rows (an edge with one end in that set is
@@ -874,14 +799,27 @@ __device__ __forceinline__ void warp_push4(const bool (&take)[4], const int (&v)
 
 // The first contraction pass, on the item's own vertices (every super-vertex
 // a single vertex, every edge weight 1).  Returns the number of phases (1:
-// everything merged; nalive: nothing did; -1 after an error); rep[i] = the smallest member of
-// i's phase, -1 if dead; the vertices in the order they were added are left
-// in D.  Keys are 16 bits (an increment past kcap is possible while several
-// threads hit one vertex, at most one per thread, so a half-word never
-// overflows into the other).
-template <typename IT>
-__device__ __forceinline__ int first_pass(const Mem<IT> &m, int32_t *rep, int n, int nalive,
-                                          int kcap, unsigned *err, Sh &sh) {
+// everything merged; nalive: nothing did; -1 after an error) and of
+// components.  rep[i] (B or A) = the smallest member of i's phase, -1 if
+// dead; the vertices in the order they were added are left in D.  A first
+// vertex of key 0 starts another component (every vertex of the one before
+// has been added); with more than one, H[i] = the smallest member of i's
+// component, -1 if dead; past MAX_COMP the pass gives up (-2).  With kcap = 1
+// the phases are the components.  Uses C, D, F, G, H and the keys.  Keys are
+// 16 bits (an increment past kcap is possible while several threads hit one
+// vertex, at most one per thread, so a half-word never overflows into the
+// other).
+//
+// Not inlined: it runs at three places of an item, and the kernel's code is
+// long enough for the instruction cache to matter.  An item in shared memory
+// is carved again here (n vertices, d entries), so that its pointers keep
+// their address space.
+template <typename IT, bool SM>
+__device__ __noinline__ int2 first_pass(const Mem<IT> *m0, int64_t d, bool rep_in_b, int n, int nalive,
+                                        int kcap, unsigned *err, Sh *shp) {
+  Sh &sh = *shp;
+  const Mem<IT> m = SM ? carve<IT>(wcc_dyn_smem, n, d) : *m0;
+  int32_t *rep = rep_in_b ? m.B : m.A;
   uint32_t *kw = m.kw;
   volatile uint16_t *kh = reinterpret_cast<volatile uint16_t *>(m.kw);
   int32_t *queue = m.D, *phmin = m.C, *lr = m.G;
@@ -896,11 +834,12 @@ __device__ __forceinline__ int first_pass(const Mem<IT> &m, int32_t *rep, int n,
   for (int i = threadIdx.x; i < n; i += RB) rep[i] = -1;
   if (threadIdx.x < 3) sh.qn[threadIdx.x] = 0;
   if (threadIdx.x == 0) sh.ntouched = 0;
-  int tail = 0, phases = 0, r = 0, rounds = 0;
+  int tail = 0, phases = 0, r = 0, rounds = 0, comps = 0, comp = -1;
   __syncthreads();
   while (tail < nalive) {
     // the phase's first vertex: largest key, then smallest id
     int X;
+    bool fresh;  // its key is 0
     if (sizeof(IT) == 2) {
       unsigned best = 0u;
       for (int w = threadIdx.x; w < nw; w += RB) {
@@ -911,6 +850,7 @@ __device__ __forceinline__ int first_pass(const Mem<IT> &m, int32_t *rep, int n,
       }
       best = block_best(best, sh);
       X = best ? (int)(0xffffu - (best & 0xffffu)) : -1;
+      fresh = (best >> 16) == 0u;
     } else {
       unsigned long long best = 0ull;
       for (int w = threadIdx.x; w < nw; w += RB) {
@@ -922,15 +862,21 @@ __device__ __forceinline__ int first_pass(const Mem<IT> &m, int32_t *rep, int n,
       }
       best = block_best(best, sh);
       X = best ? (int)~(unsigned)best : -1;
+      fresh = (best >> 32) == 0ull;
     }
     if (X < 0 || X >= n) {  // cannot happen: an unadded vertex has a key below kcap here
       if (threadIdx.x == 0) atomicOr(err, DERR_INTERNAL);
-      return -1;
+      return make_int2(-1, 0);
+    }
+    if (fresh) {
+      comp = X;
+      if (++comps > MAX_COMP) return make_int2(-2, 0);
     }
     if (threadIdx.x == 0) {
       queue[tail] = X;
       rep[X] = phases;
       phmin[phases] = X;
+      m.F[phases] = comp;
       kh[X] = (uint16_t)KEY_IN;
     }
     int head = tail++;
@@ -1054,10 +1000,11 @@ __device__ __forceinline__ int first_pass(const Mem<IT> &m, int32_t *rep, int n,
   }
   for (int i = threadIdx.x; i < n; i += RB) {
     const int p = rep[i];
+    if (comps > 1) m.H[i] = p >= 0 ? m.F[p] : -1;
     if (p >= 0) rep[i] = phmin[p];
   }
   __syncthreads();
-  return phases;
+  return make_int2(phases, comps);
 }
 
 // A later pass, on super-vertices with members (rep[i] = the smallest member
@@ -2224,7 +2171,9 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
 
   // 2. input cluster: CCR (Algorithm 1)
   if (it.flags & ITEM_TOP) {
-    int nc = components_af(m, n, m.B, m.H, sh);
+    int nc = first_pass<IT, SM>(&m, dbound, true, n, n, 1, &P.ctr->error, &sh).x;
+    if (nc == -1) return OUT_ERROR;
+    if (nc == -2) nc = components_af(m, n, m.B, m.H, sh);
     if (nc != 1) {
       int emitted = 0;
       const int L = emit_children(P, R, Rg, it.req, m, m.B, n, vb, sh, 0, true, &emitted);
@@ -2236,28 +2185,68 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
   }
   prof_stamp(P, sh, 3);
 
-  // 3. peel (round-synchronous, T recomputed from the alive count)
+  // 3. peel (round-synchronous, T recomputed from the alive count).  T never
+  // grows, so after the first round only a vertex whose degree has just
+  // dropped to T can go: each drop to T lists it once, and the next round
+  // takes the listed ones that its own T still covers (the others are listed
+  // again when they drop to it).
   int32_t *deg = m.A;
-  for (int i = threadIdx.x; i < n; i += RB) deg[i] = (int32_t)m.len[i];
-  __syncthreads();
   const int n_item = nalive;
-  for (;;) {
-    const int64_t T = threshold_of(R.rule_kind, R.rule_num, R.rule_den, nalive);
-    int rem = 0;
-    for (int i = threadIdx.x; i < n; i += RB) {
-      bool r = m.alive[i] && deg[i] <= T;
-      m.flag[i] = r;
-      rem += r;
-    }
-    rem = block_sum_int(rem, sh);
-    if (rem == 0) break;
-    for (int i = warp; i < n; i += RW) {
-      if (!m.flag[i]) continue;
-      for (int e = m.off[i] + lane; e < m.end(i); e += 32) atomicSub(&deg[m.adj[e]], 1);
-      if (lane == 0) m.alive[i] = 0;
+  {
+    int32_t *cand = m.G, *next = m.H;
+    int64_t T = threshold_of(R.rule_kind, R.rule_num, R.rule_den, nalive);
+    if (threadIdx.x < 3) sh.qn[threadIdx.x] = 0;
+    __syncthreads();
+    for (int i0 = 0; i0 < n; i0 += RB) {
+      const int i = i0 + threadIdx.x;
+      int d = 0;
+      if (i < n) deg[i] = d = (int)m.len[i];
+      warp_push(i < n && m.alive[i] && d <= T, i, cand, 0, &sh.qn[0]);
     }
     __syncthreads();
-    nalive -= rem;
+    int nc = *(volatile int32_t *)&sh.qn[0];
+    for (int r = 1; nc > 0; r = r == 2 ? 0 : r + 1) {
+      T = threshold_of(R.rule_kind, R.rule_num, R.rule_den, nalive);
+      int rem = 0;
+      for (int q = threadIdx.x; q < nc; q += RB) {
+        const int i = cand[q];
+        if (deg[i] <= T) {
+          m.alive[i] = 0;
+          ++rem;
+        } else {
+          cand[q] = -1;
+        }
+      }
+      if (threadIdx.x == 0) sh.qn[r == 2 ? 0 : r + 1] = 0;
+      rem = block_sum_int(rem, sh);
+      if (rem == 0) break;
+      nalive -= rem;
+      const int per = min(32, (nc + RW - 1) / RW);
+      for (int c0 = warp * per; c0 < nc; c0 += RW * per) {
+        int b = 0, d = 0, exc;
+        if (lane < min(per, nc - c0)) {
+          const int i = cand[c0 + lane];
+          if (i >= 0) {
+            b = m.off[i];
+            d = (int)m.len[i];
+          }
+        }
+        flat_rows(m.adj, b, d, exc, [&](const int (&j)[4], int) {
+          bool drop[4];
+#pragma unroll
+          for (int z = 0; z < 4; ++z) drop[z] = j[z] >= 0 && m.alive[j[z]];
+#pragma unroll
+          for (int z = 0; z < 4; ++z)
+            if (drop[z]) drop[z] = (int64_t)atomicSub(&deg[j[z]], 1) - 1 == T;
+          warp_push4(drop, j, next, 0, &sh.qn[r]);
+        });
+      }
+      __syncthreads();
+      nc = *(volatile int32_t *)&sh.qn[r];
+      int32_t *t = cand;
+      cand = next;
+      next = t;
+    }
   }
   if (threadIdx.x == 0) {
     if (nalive < n_item) add_ll(&ctr->peeled, (long long)(n_item - nalive));
@@ -2269,17 +2258,47 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
   // 4. connectivity of what is left (an item arrives connected: input
   // clusters passed CCR above, children are components or sides of a
   // minimum cut, which are connected; only a peel can disconnect it).  The
-  // component continued in place needs no peel of its own: T only grows
-  // with n, so every vertex left already has degree > T of its smaller size.
+  // first contraction pass of step 5 finds the components on its way: it
+  // runs here, and stands for the component continued in place too (no edge
+  // joins the components, so that one's phases are those it has alone) unless
+  // its smaller size changes T.  That component needs no peel of its own: T
+  // only grows with n, so every vertex left already has degree > T of its
+  // smaller size.
+  int32_t *rep = m.A;
+  int pre = 0;             // > 0: sets of the first pass, which has run already
+  bool pre_order = false;  // ... and the order of adding is in D
   if (nalive < n_item) {
-    int nc = components_af(m, n, m.B, m.H, sh);
-    if (nc > 1) {
+    const int64_t T0 = threshold_of(R.rule_kind, R.rule_num, R.rule_den, nalive);
+    int comps = 0, ph = -2;
+    const int32_t *label = m.H;
+    if (T0 < KEY_MAX) {
+      const int2 r = first_pass<IT, SM>(&m, dbound, false, n, nalive, (int)T0 + 1, &P.ctr->error, &sh);
+      ph = r.x;
+      comps = r.y;
+    }
+    if (ph == -1) return OUT_ERROR;
+    if (ph == -2) {
+      comps = components_af(m, n, m.B, m.H, sh);
+      label = m.B;
+    }
+    if (comps > 1) {
       int emitted = 0;
-      const int L = emit_children(P, R, Rg, it.req, m, m.B, n, vb, sh, 0, true, &emitted);
+      const int L = emit_children(P, R, Rg, it.req, m, label, n, vb, sh, 0, true, &emitted);
       if (L < 0) return OUT_CC_SPLIT;
-      nalive = restrict_alive(m, m.B, L, n, sh);
+      nalive = restrict_alive(m, label, L, n, sh);
       vb += emitted;
       if (threadIdx.x == 0) add_ll(&ctr->items, 1ll);
+      if (ph > 0 && threshold_of(R.rule_kind, R.rule_num, R.rule_den, nalive) == T0) {
+        int r1 = 0;
+        for (int i = threadIdx.x; i < n; i += RB) {
+          if (!m.alive[i]) rep[i] = -1;
+          r1 += rep[i] == i;
+        }
+        pre = block_sum_int(r1, sh);
+      }
+    } else if (ph > 0) {
+      pre = ph;
+      pre_order = true;
     }
   }
   prof_stamp(P, sh, 5);
@@ -2287,7 +2306,6 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
   // 5. contraction with k = T+1
   const int64_t T = threshold_of(R.rule_kind, R.rule_num, R.rule_den, nalive);
   const int kcap = (int)(T + 1 < (1ll << 30) ? T + 1 : (1ll << 30));
-  int32_t *rep = m.A;
   int nsv = 1, passes = 0;
   int dense_cut = -1;  // >= 0: the dense finish found the cut (side in m.side)
   bool certified = false;
@@ -2302,6 +2320,7 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
       cf = reinterpret_cast<int32_t *>(wcc_dyn_smem);
     const int fr = forest_accept(m, n, kcap, cf, sh, P.prof != nullptr);
     certified = fr > 0;
+    pre_order = false;
     if (P.prof && threadIdx.x == 0) {
       sh.pf_forest = fr;
       sh.pf_forest_cycles = clock64() - f0;
@@ -2352,11 +2371,19 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
         inh_valid = true;
       } else {
         const long long p0 = P.prof ? clock64() : 0;
-        nsv = first_pass(m, rep, n, nalive, kcap, &P.ctr->error, sh);
-        if (nsv < 0) return OUT_ERROR;
+        if (pre > 0) {
+          nsv = pre;
+        } else {
+          // (what is left is connected)
+          nsv = first_pass<IT, SM>(&m, dbound, false, n, nalive, kcap, &P.ctr->error, &sh).x;
+          if (nsv < 0) {
+            if (threadIdx.x == 0) atomicOr(&P.ctr->error, DERR_INTERNAL);
+            return OUT_ERROR;
+          }
+        }
         // this pass's records, for the sides of a later cut (the order of
         // adding is in D)
-        inh_valid = R.inh != nullptr && recordable && nalive >= INH_MIN_N;
+        inh_valid = R.inh != nullptr && recordable && nalive >= INH_MIN_N && (pre == 0 || pre_order);
         if (inh_valid) {
           for (int q = threadIdx.x; q < nalive; q += RB) {
             const int i = m.D[q];
