@@ -35,7 +35,13 @@ namespace wccg {
 
 namespace {
 
-constexpr int RB = 256;        // threads per CTA
+// Threads per CTA, one CTA per SM.  The block-wide loops are bound by latency,
+// so more warps hide more of it, until 128 registers a thread are too few and
+// a barrier costs more than it saves.  Graph resident, with 256 / 512 / 1024
+// threads: clusters of up to 50,000 vertices (1M vertices) 8.96 / 6.78 / 6.20
+// ms, small clusters (2M) 4.28 / 3.98 / 4.21, LFR-style 100k 0.567 / 0.557 /
+// 0.593, planted 1k 0.246 / 0.255 / 0.283.
+constexpr int RB = 512;
 constexpr int RW = RB / 32;    // warps per CTA
 constexpr size_t SMEM_MAX_BYTES = 227 * 1024;  // opt-in limit per CTA
 
@@ -138,6 +144,13 @@ __device__ __forceinline__ bool carve_hot(Mem<IT> &m, int n, size_t smem_bytes) 
   return true;
 }
 
+// The item's memory in a function that is not inlined: an item in shared
+// memory is carved again, so that its pointers keep their address space.
+template <typename IT, bool SM>
+__device__ __forceinline__ Mem<IT> item_mem(const Mem<IT> *m0, int n, int64_t d) {
+  return SM ? carve<IT>(wcc_dyn_smem, n, d) : *m0;
+}
+
 // Block-level scalars.
 struct Sh {
   int32_t scan[RW + 1];
@@ -167,7 +180,6 @@ struct Sh {
   unsigned long long cta_seq[TINY_BLOCK + 1];
   unsigned long long tst[7];   // statistics of the batch's small items
   int32_t duf[32];    // dense finish: merges of one pass (union-find over indices)
-  uint32_t dside;     // dense finish: side of the minimum cut (mask of indices)
   int32_t wduf[128], wgrp[128];  // wide dense finish: union-find, sets of initial indices
   uint32_t wside[4];             // wide dense finish: side of the minimum cut
   int32_t dcut, dpasses, dphases;
@@ -368,11 +380,13 @@ __device__ __forceinline__ void afforest(const Mem<IT> &m, int n, int32_t *uf, i
   __syncthreads();
 }
 
-// Connected components of the alive vertices by afforest(): f[i] = smallest
+// Connected components of the alive vertices by afforest(): B[i] = smallest
 // alive id of i's component (-1 if dead); returns the number of components.
-template <typename IT>
-__device__ __forceinline__ int components_af(const Mem<IT> &m, int n, int32_t *f, int32_t *cur,
-                                             Sh &sh) {
+template <typename IT, bool SM>
+__device__ __noinline__ int components_af(const Mem<IT> *m0, int64_t d, int n, Sh *shp) {
+  Sh &sh = *shp;
+  const Mem<IT> m = item_mem<IT, SM>(m0, n, d);
+  int32_t *f = m.B, *cur = m.H;
   afforest(m, n, f, cur, sh);
   int roots = 0;
   for (int i = threadIdx.x; i < n; i += RB) {
@@ -387,19 +401,27 @@ __device__ __forceinline__ int components_af(const Mem<IT> &m, int n, int32_t *f
 }
 
 // ---- publishing children -------------------------------------------------
-// tag[i] in [0, n) names the child of local vertex i (-1: none).  Every tag
+// tag[i] (B or H) in [0, n) names the child of local vertex i (-1: none).  Every tag
 // with at least min_size members becomes a new queue item whose vertex list
 // (ascending) is written into the parent's pool range.  Uses C, D, E, F.
 // With keep_largest, the kept child with the most members (ties: smallest
 // tag) is not published: the caller refines it in place, and the children
 // that are published fill the front of the range.  Returns that child's tag
 // (-1: none) and, in *emitted, the members published ahead of it.
-template <typename IT>
-__device__ __forceinline__ int emit_children(const RefineParams &P, const ReqCtx &R,
-                                             ReqCtx *Rg, uint16_t req, const Mem<IT> &m,
-                                             const int32_t *tag, int n, int64_t vbeg, Sh &sh,
-                                             uint16_t cflags = 0, bool keep_largest = false,
-                                             int *emitted = nullptr) {
+//
+// This and the other parts of an item that are rare, long or used at several
+// places are not inlined (item_mem says how they find the item's memory): the
+// kernel's code then fits the instruction cache better and its main path the
+// registers of 512 threads.
+enum : int { TAG_B = 0, TAG_H = 1 };
+template <typename IT, bool SM>
+__device__ __noinline__ int emit_children(const RefineParams &P, const ReqCtx &R, ReqCtx *Rg,
+                                          uint16_t req, const Mem<IT> *m0, int64_t d, int which,
+                                          int n, int64_t vbeg, Sh *shp, uint16_t cflags = 0,
+                                          bool keep_largest = false, int *emitted = nullptr) {
+  Sh &sh = *shp;
+  const Mem<IT> m = item_mem<IT, SM>(m0, n, d);
+  const int32_t *tag = which == TAG_H ? m.H : m.B;
   int32_t *cnt = m.C, *cidx = m.D, *cbase = m.E, *run = m.F;
   for (int t = threadIdx.x; t < n; t += RB) cnt[t] = 0;
   if (threadIdx.x == 0) sh.u1 = 0ull;
@@ -698,9 +720,9 @@ constexpr unsigned KEY_IN = 0x8000u;    // added, or queued to be
 constexpr unsigned KEY_DEAD = 0x4000u;  // peeled: never below kcap, never added
 constexpr int KEY_MAX = 0x3fff;         // largest kcap the 16-bit keys hold
 // A round looks from the unadded vertices' side when the vertices added in
-// the round before are at least twice as many: the last rounds add most of
-// the vertices at once, and an unadded one stops at kcap added neighbours,
-// most often within its first 32 entries.
+// the round before are at least as many: the last rounds add most of the
+// vertices at once, and an unadded one stops at kcap added neighbours, most
+// often within its first 32 entries.
 constexpr int PULL_MIN = 64;
 constexpr int PULL_STEP = 32;
 
@@ -809,16 +831,11 @@ __device__ __forceinline__ void warp_push4(const bool (&take)[4], const int (&v)
 // 16 bits (an increment past kcap is possible while several threads hit one
 // vertex, at most one per thread, so a half-word never overflows into the
 // other).
-//
-// Not inlined: it runs at three places of an item, and the kernel's code is
-// long enough for the instruction cache to matter.  An item in shared memory
-// is carved again here (n vertices, d entries), so that its pointers keep
-// their address space.
 template <typename IT, bool SM>
 __device__ __noinline__ int2 first_pass(const Mem<IT> *m0, int64_t d, bool rep_in_b, int n, int nalive,
                                         int kcap, unsigned *err, Sh *shp) {
   Sh &sh = *shp;
-  const Mem<IT> m = SM ? carve<IT>(wcc_dyn_smem, n, d) : *m0;
+  const Mem<IT> m = item_mem<IT, SM>(m0, n, d);
   int32_t *rep = rep_in_b ? m.B : m.A;
   uint32_t *kw = m.kw;
   volatile uint16_t *kh = reinterpret_cast<volatile uint16_t *>(m.kw);
@@ -886,7 +903,7 @@ __device__ __noinline__ int2 first_pass(const Mem<IT> *m0, int64_t d, bool rep_i
       int32_t *qn = &sh.qn[r];
       const int rn = r == 2 ? 0 : r + 1;
       if (threadIdx.x == 0) sh.qn[rn] = 0;
-      if (F >= PULL_MIN && F >= 2 * U) {
+      if (F >= PULL_MIN && F >= U) {
         // every unadded vertex counts its added neighbours afresh; those it
         // takes are marked only after the round, so that the keys of the
         // rest are exact
@@ -1007,13 +1024,17 @@ __device__ __noinline__ int2 first_pass(const Mem<IT> *m0, int64_t d, bool rep_i
   return make_int2(phases, comps);
 }
 
-// A later pass, on super-vertices with members (rep[i] = the smallest member
-// of i's set): the same phases, keys counting the edges of all members.
-// Needs group_members(m, rep).  Returns the number of phases (-1 after an
-// error) and moves rep to their sets.  Uses B, E, F, H.
-template <typename IT>
-__device__ __forceinline__ int class_pass(const Mem<IT> &m, int32_t *rep, int n, int nsv, int kcap,
-                                          unsigned *err, Sh &sh) {
+// A later pass, on super-vertices with members (rep[i], in A, = the smallest
+// member of i's set): the same phases, keys counting the edges of all
+// members.  Returns the number of phases (-1 after an error) and moves rep
+// to their sets.  Uses B, C, D, E, F, G, H.
+template <typename IT, bool SM>
+__device__ __noinline__ int class_pass(const Mem<IT> *m0, int64_t d, int n, int kcap,
+                                       unsigned *err, Sh *shp) {
+  Sh &sh = *shp;
+  const Mem<IT> m = item_mem<IT, SM>(m0, n, d);
+  int32_t *rep = m.A;
+  const int nsv = group_members(m, rep, n, sh);
   constexpr unsigned IN = 0x80000000u;
   unsigned *key = reinterpret_cast<unsigned *>(m.F);
   volatile unsigned *vkey = key;
@@ -1165,6 +1186,48 @@ __device__ __forceinline__ void ma_ordering_block(const Mem<IT> &m, const int32_
   __syncthreads();
 }
 
+template <typename IT>
+__device__ __forceinline__ void reset_ma_state(const Mem<IT> &m, int n) {
+  for (int i = threadIdx.x; i < n; i += RB) {
+    m.E[i] = 0;
+    m.F[i] = 0;
+    m.flag[i] = 0;
+  }
+  __syncthreads();
+}
+
+// Canonical Stoer-Wagner over the sets grp (in A), phase by phase: the first
+// smallest cut of a phase, its side in m.side; *phases counts them.
+template <typename IT, bool SM>
+__device__ __noinline__ int sparse_cut(const Mem<IT> *m0, int64_t d, int n, int nsv,
+                                       long long *phases, Sh *shp) {
+  Sh &sh = *shp;
+  const Mem<IT> m = item_mem<IT, SM>(m0, n, d);
+  int32_t *grp = m.A;
+  int best = 0x7fffffff;
+  while (nsv > 1) {
+    group_members(m, grp, n, sh);
+    reset_ma_state(m, n);
+    if (threadIdx.x == 0) add_ll(phases, 1ll);
+    if (nsv <= BLOCK_NSV)
+      ma_ordering_block(m, grp, nsv, sh);
+    else
+      ma_ordering(m, grp, nsv, sh);
+    const int s = sh.sw_s, t = sh.sw_t, cut = sh.sw_cut;
+    if (cut < best) {
+      best = cut;
+      for (int i = threadIdx.x; i < n; i += RB) m.side[i] = m.alive[i] && grp[i] == t;
+    }
+    __syncthreads();
+    const int lo = s < t ? s : t, hi = s < t ? t : s;
+    for (int i = threadIdx.x; i < n; i += RB)
+      if (m.alive[i] && grp[i] == hi) grp[i] = lo;
+    __syncthreads();
+    --nsv;
+  }
+  return best;
+}
+
 // ---- few super-vertices: a dense finish ---------------------------------------
 // With at most 32 super-vertices left (indexed in ascending order of their
 // smallest member, so index order is id order), their integer edge weights
@@ -1241,7 +1304,7 @@ struct DenseResult {
 // Runs the dense finish on w (nsv <= 32 indices; the super-vertices are the
 // indices in live0) with one warp (any warp; all its lanes call).  duf: 32
 // ints of scratch.  Every lane returns the result.
-__device__ DenseResult dense_finish(int32_t *w, int nsv, uint32_t live0, int kcap, int32_t *duf) {
+__device__ __forceinline__ DenseResult dense_finish(int32_t *w, int nsv, uint32_t live0, int kcap, int32_t *duf) {
   const int l = threadIdx.x & 31;
   uint32_t live = live0;
   uint32_t mem = 1u << l;  // lane l: the initial indices it holds
@@ -1397,7 +1460,7 @@ __device__ __forceinline__ void dense_order_w(const int32_t *w, int nsv, const u
 
 // duf, grp: nsv ints each; side: K words.
 template <int K>
-__device__ DenseResult dense_finish_w(int32_t *w, int nsv, int kcap, int32_t *duf, int32_t *grp,
+__device__ __noinline__ DenseResult dense_finish_w(int32_t *w, int nsv, int kcap, int32_t *duf, int32_t *grp,
                                       uint32_t *side) {
   const int l = threadIdx.x & 31;
   uint32_t live[K];
@@ -1457,6 +1520,26 @@ __device__ DenseResult dense_finish_w(int32_t *w, int nsv, int kcap, int32_t *du
   return res;
 }
 
+// The dense finish of a CTA's item, by its first warp; w: nsv x nsv weights.
+// The result and the cut's side are left in sh for the other warps.
+__device__ __noinline__ void dense_cta(int32_t *w, int nsv, int kcap, Sh *shp) {
+  Sh &sh = *shp;
+  DenseResult dr;
+  if (nsv <= DENSE_NSV) {
+    dr = dense_finish(w, nsv, nsv >= 32 ? 0xffffffffu : (1u << nsv) - 1u, kcap, sh.duf);
+    if (threadIdx.x == 0) sh.wside[0] = dr.side;
+  } else if (nsv <= 64) {
+    dr = dense_finish_w<2>(w, nsv, kcap, sh.wduf, sh.wgrp, sh.wside);
+  } else {
+    dr = dense_finish_w<4>(w, nsv, kcap, sh.wduf, sh.wgrp, sh.wside);
+  }
+  if (threadIdx.x == 0) {
+    sh.dcut = dr.cut;
+    sh.dpasses = dr.passes;
+    sh.dphases = dr.phases;
+  }
+}
+
 // Exact acceptance test for lambda >= kcap by forest certificates.  Take
 // kcap-1 edge-disjoint spanning forests, each maximal in the edges the earlier
 // ones left.  An edge (u, v) in none of them has u and v joined by a path in
@@ -1504,8 +1587,10 @@ __device__ __forceinline__ void rows_pass(const Mem<IT> &m, int n, const int32_t
 }
 
 template <typename IT>
-__device__ __forceinline__ int forest_accept(const Mem<IT> &m, int n, int kcap, int32_t *cf, Sh &sh,
-                                             bool prof) {
+__device__ __noinline__ int forest_accept(const Mem<IT> *m0, int n, int kcap, int32_t *cf, Sh *shp,
+                                          bool prof) {
+  Sh &sh = *shp;
+  const Mem<IT> m = *m0;
   long long tc = prof ? clock64() : 0;
   auto lap = [&](int k) {  // profile: cycles since the last lap into fdbg[k]
     if (prof) {
@@ -1598,33 +1683,13 @@ __device__ __forceinline__ int forest_accept(const Mem<IT> &m, int n, int kcap, 
         if (B >= 0 && B != A) atomicAdd(&w[idx[A] * nroots + idx[B]], 1);
       });
       __syncthreads();
-      if (threadIdx.x < 32) {
-        DenseResult dr;
-        if (nroots <= DENSE_NSV)
-          dr = dense_finish(w, nroots, nroots >= 32 ? 0xffffffffu : (1u << nroots) - 1u, kcap,
-                            sh.duf);
-        else if (nroots <= 64)
-          dr = dense_finish_w<2>(w, nroots, kcap, sh.wduf, sh.wgrp, sh.wside);
-        else
-          dr = dense_finish_w<4>(w, nroots, kcap, sh.wduf, sh.wgrp, sh.wside);
-        if (threadIdx.x == 0) sh.dcut = dr.cut;
-      }
+      if (threadIdx.x < 32) dense_cta(w, nroots, kcap, &sh);
       __syncthreads();
       lap(3);
       return sh.dcut < 0 ? round : -round;
     }
   }
   return -FOREST_ROUNDS;
-}
-
-template <typename IT>
-__device__ __forceinline__ void reset_ma_state(const Mem<IT> &m, int n) {
-  for (int i = threadIdx.x; i < n; i += RB) {
-    m.E[i] = 0;
-    m.F[i] = 0;
-    m.flag[i] = 0;
-  }
-  __syncthreads();
 }
 
 // ---- items of at most 64 vertices: one warp each ---------------------------------
@@ -2173,10 +2238,11 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
   if (it.flags & ITEM_TOP) {
     int nc = first_pass<IT, SM>(&m, dbound, true, n, n, 1, &P.ctr->error, &sh).x;
     if (nc == -1) return OUT_ERROR;
-    if (nc == -2) nc = components_af(m, n, m.B, m.H, sh);
+    if (nc == -2) nc = components_af<IT, SM>(&m, dbound, n, &sh);
     if (nc != 1) {
       int emitted = 0;
-      const int L = emit_children(P, R, Rg, it.req, m, m.B, n, vb, sh, 0, true, &emitted);
+      const int L = emit_children<IT, SM>(P, R, Rg, it.req, &m, dbound, TAG_B, n, vb, &sh, 0, true,
+                                              &emitted);
       if (L < 0) return OUT_CCR_SPLIT;
       nalive = restrict_alive(m, m.B, L, n, sh);
       vb += emitted;
@@ -2270,22 +2336,21 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
   if (nalive < n_item) {
     const int64_t T0 = threshold_of(R.rule_kind, R.rule_num, R.rule_den, nalive);
     int comps = 0, ph = -2;
-    const int32_t *label = m.H;
-    if (T0 < KEY_MAX) {
+        if (T0 < KEY_MAX) {
       const int2 r = first_pass<IT, SM>(&m, dbound, false, n, nalive, (int)T0 + 1, &P.ctr->error, &sh);
       ph = r.x;
       comps = r.y;
     }
     if (ph == -1) return OUT_ERROR;
     if (ph == -2) {
-      comps = components_af(m, n, m.B, m.H, sh);
-      label = m.B;
+      comps = components_af<IT, SM>(&m, dbound, n, &sh);
     }
     if (comps > 1) {
       int emitted = 0;
-      const int L = emit_children(P, R, Rg, it.req, m, label, n, vb, sh, 0, true, &emitted);
+      const int L = emit_children<IT, SM>(P, R, Rg, it.req, &m, dbound, ph == -2 ? TAG_B : TAG_H, n, vb,
+                                              &sh, 0, true, &emitted);
       if (L < 0) return OUT_CC_SPLIT;
-      nalive = restrict_alive(m, label, L, n, sh);
+      nalive = restrict_alive(m, ph == -2 ? m.B : m.H, L, n, sh);
       vb += emitted;
       if (threadIdx.x == 0) add_ll(&ctr->items, 1ll);
       if (ph > 0 && threshold_of(R.rule_kind, R.rule_num, R.rule_den, nalive) == T0) {
@@ -2318,7 +2383,7 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
     int32_t *cf = m.B;
     if (!SM && !m.off_in_smem && 4 * (size_t)n <= P.smem_bytes)
       cf = reinterpret_cast<int32_t *>(wcc_dyn_smem);
-    const int fr = forest_accept(m, n, kcap, cf, sh, P.prof != nullptr);
+    const int fr = forest_accept(&m, n, kcap, cf, &sh, P.prof != nullptr);
     certified = fr > 0;
     pre_order = false;
     if (P.prof && threadIdx.x == 0) {
@@ -2415,10 +2480,9 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
         }
       }
       if (wmat == nullptr) {  // another pass on the sets
-        nsv = group_members(m, rep, n, sh);
         if (threadIdx.x == 0) add_ll(&ctr->ni_passes, 1ll);
         ++passes;
-        const int k = class_pass(m, rep, n, nsv, kcap, &P.ctr->error, sh);
+        const int k = class_pass<IT, SM>(&m, dbound, n, kcap, &P.ctr->error, &sh);
         if (k < 0) return OUT_ERROR;
         more = k < nsv;
         nsv = k;
@@ -2481,23 +2545,7 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
         }
       }
       __syncthreads();
-      if (threadIdx.x < 32) {
-        DenseResult dr;
-        if (nsv <= DENSE_NSV) {
-          dr = dense_finish(w, nsv, nsv >= 32 ? 0xffffffffu : (1u << nsv) - 1u, kcap, sh.duf);
-          if (threadIdx.x == 0) sh.wside[0] = dr.side;
-        } else if (nsv <= 64) {
-          dr = dense_finish_w<2>(w, nsv, kcap, sh.wduf, sh.wgrp, sh.wside);
-        } else {
-          dr = dense_finish_w<4>(w, nsv, kcap, sh.wduf, sh.wgrp, sh.wside);
-        }
-        if (threadIdx.x == 0) {
-          sh.dcut = dr.cut;
-          sh.dside = dr.side;
-          sh.dpasses = dr.passes;
-          sh.dphases = dr.phases;
-        }
-      }
+      if (threadIdx.x < 32) dense_cta(w, nsv, kcap, &sh);
       __syncthreads();
       passes += sh.dpasses;
       if (threadIdx.x == 0) {
@@ -2545,28 +2593,7 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
       return OUT_ERROR;
     }
   } else {
-    int32_t *grp = m.A;
-    int best = 0x7fffffff;
-    while (nsv > 1) {
-      group_members(m, grp, n, sh);
-      reset_ma_state(m, n);
-      if (threadIdx.x == 0) add_ll(&ctr->sw_phases, 1ll);
-      if (nsv <= BLOCK_NSV)
-        ma_ordering_block(m, grp, nsv, sh);
-      else
-        ma_ordering(m, grp, nsv, sh);
-      const int s = sh.sw_s, t = sh.sw_t, cut = sh.sw_cut;
-      if (cut < best) {
-        best = cut;
-        for (int i = threadIdx.x; i < n; i += RB) m.side[i] = m.alive[i] && grp[i] == t;
-      }
-      __syncthreads();
-      const int lo = s < t ? s : t, hi = s < t ? t : s;
-      for (int i = threadIdx.x; i < n; i += RB)
-        if (m.alive[i] && grp[i] == hi) grp[i] = lo;
-      __syncthreads();
-      --nsv;
-    }
+    const int best = sparse_cut<IT, SM>(&m, dbound, n, nsv, &ctr->sw_phases, &sh);
     prof_stamp(P, sh, 7);
     if (best > T) {
       if (threadIdx.x == 0) atomicOr(&P.ctr->error, DERR_INTERNAL);
@@ -2579,7 +2606,8 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
   if (P.cm)
     park_sides(P, R, it.req, m, m.B, n, vb, sh);
   else
-    emit_children(P, R, Rg, it.req, m, m.B, n, vb, sh, inh_valid ? ITEM_INH : (uint16_t)0);
+    emit_children<IT, SM>(P, R, Rg, it.req, &m, dbound, TAG_B, n, vb, &sh,
+                          inh_valid ? ITEM_INH : (uint16_t)0);
   return OUT_CUT_SPLIT;
 }
 
