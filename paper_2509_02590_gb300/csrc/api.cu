@@ -186,17 +186,13 @@ int tiny_max_deg_config() {
   return (int)(v < 0 ? 0 : v > (1ll << 30) ? (1ll << 30) : v);
 }
 
-// CSR builder of wcc_create_graph_from_edges (WCC_CSR_BUILDER): "rows" sorts
-// every row on chip (and sorts all entries at once when a row is too long
-// for that); "radix" always sorts all entries at once; "auto" (the default)
-// takes the rows for edge lists of up to CSR_ROWS_AUTO_MAX_EDGES edges.  Both
-// give the same CSR.
-constexpr int64_t CSR_ROWS_AUTO_MAX_EDGES = 1ll << 24;
-bool csr_rows_config(int64_t m) {
+// CSR builder of wcc_create_graph_from_edges (WCC_CSR_BUILDER): "radix" sorts
+// all entries at once; "rows" and "auto" (the default) partition them into
+// buckets of rows sorted on chip and sort all entries at once only when a
+// graph does not fit that (see csr_by_buckets).  All give the same CSR.
+bool csr_buckets_config() {
   const char *e = getenv("WCC_CSR_BUILDER");
-  if (e && strcmp(e, "rows") == 0) return true;
-  if (e && strcmp(e, "radix") == 0) return false;
-  return m <= CSR_ROWS_AUTO_MAX_EDGES;
+  return !(e && strcmp(e, "radix") == 0);
 }
 
 // Dynamic shared memory per refinement CTA (WCC_SMEM_KB, default: the
@@ -641,9 +637,9 @@ Graph *build_from_edges(const int32_t *src, const int32_t *dst, int64_t m, int64
   int64_t *d_off = static_cast<int64_t *>(g->off.ensure(8 * (n + 1)));
   WCC_CUDA(cudaMemsetAsync(d_off, 0, 8 * (n + 1), s));
   int64_t nnz = 0;
-  if (m > 0 && csr_rows_config(m)) {
-    DevBuf rbufs[CSR_ROW_BUFS];
-    if (csr_by_rows(d_src, d_dst, m, n, d_off, g->adj, &nnz, rbufs, s)) {
+  if (m > 0 && csr_buckets_config()) {
+    DevBuf bufs[CSR_BUCKET_BUFS];
+    if (csr_by_buckets(d_src, d_dst, m, n, d_off, g->adj, &nnz, bufs, s)) {
       g->nnz = nnz;
       return g.release();
     }
