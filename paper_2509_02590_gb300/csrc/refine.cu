@@ -179,9 +179,8 @@ struct Sh {
   Item cta_item[TINY_BLOCK + 1];
   unsigned long long cta_seq[TINY_BLOCK + 1];
   unsigned long long tst[7];   // statistics of the batch's small items
-  int32_t duf[32];    // dense finish: merges of one pass (union-find over indices)
-  int32_t wduf[128], wgrp[128];  // wide dense finish: union-find, sets of initial indices
-  uint32_t wside[4];             // wide dense finish: side of the minimum cut
+  int32_t wgrp[128];  // dense finish: the index that holds each initial one
+  uint32_t wside[4];  // dense finish: side of the minimum cut (mask of indices)
   int32_t dcut, dpasses, dphases;
 };
 
@@ -1229,315 +1228,247 @@ __device__ __noinline__ int sparse_cut(const Mem<IT> *m0, int64_t d, int n, int 
 }
 
 // ---- few super-vertices: a dense finish ---------------------------------------
-// With at most 32 super-vertices left (indexed in ascending order of their
+// With at most 128 super-vertices left (indexed in ascending order of their
 // smallest member, so index order is id order), their integer edge weights
 // fit a small matrix w[nsv][nsv] and one warp runs the remaining capped
 // contraction passes and the Stoer-Wagner phases on it, lane l holding
-// super-vertex l, with exactly the rules of the sparse passes: largest key,
-// ties to the smallest id; in a capped pass every X-Y whose key reaches kcap
-// when X is added merges (survivor: the smaller id); a phase's cut is the key
-// of the last super-vertex t, the earliest minimum is kept, its side is t's
-// members, and t merges into the one added before it.
-constexpr int DENSE_NSV = 32;  // one lane per super-vertex
-static_assert(DENSE_NSV <= 32, "the dense finish keeps one super-vertex per lane");
+// super-vertices l, l + 32, ... (K of them), with exactly the rules of the
+// sparse passes: largest key, ties to the smallest id; a capped pass merges
+// its phases (see "contraction passes"; survivor: the smallest id); a
+// Stoer-Wagner phase's cut is the key of the last super-vertex t, the earliest
+// minimum is kept, its side is t's members, and t merges into the one added
+// before it.  Sets of indices are bit masks, bit l of word j = index l + 32 j,
+// the same in every lane.  (With a capped pass as an ordering, one pick and
+// its union-find links a super-vertex, 67 of them took 1,500 cycles a pick and
+// the dense finish 0.29M of an item's 0.71M cycles; as phases it takes 0.09M.)
+constexpr int DENSE_NSV = 128;
 
-// Adds row and column l of w into r (r < l), zeroes r's diagonal.  Warp 0.
-__device__ __forceinline__ void dense_fold(int32_t *w, int nsv, int r, int l) {
-  const int c = threadIdx.x & 31;
-  if (c < nsv) w[r * nsv + c] += w[l * nsv + c];
+template <int K>
+struct Mask {
+  uint32_t w[K];
+  __device__ __forceinline__ bool any() const {
+    uint32_t r = 0u;
+#pragma unroll
+    for (int j = 0; j < K; ++j) r |= w[j];
+    return r != 0u;
+  }
+  __device__ __forceinline__ int count() const {
+    int r = 0;
+#pragma unroll
+    for (int j = 0; j < K; ++j) r += __popc(w[j]);
+    return r;
+  }
+  __device__ __forceinline__ int first() const {  // -1: none
+    int r = -1;
+#pragma unroll
+    for (int j = K - 1; j >= 0; --j) r = w[j] ? 32 * j + __ffs(w[j]) - 1 : r;
+    return r;
+  }
+  __device__ __forceinline__ void clear(int x) {
+#pragma unroll
+    for (int j = 0; j < K; ++j) w[j] &= (x >> 5) == j ? ~(1u << (x & 31)) : FULL;
+  }
+  __device__ __forceinline__ bool mine(int j) const { return (w[j] >> (threadIdx.x & 31)) & 1u; }
+};
+
+// Folds the rows and columns of the indices in C into its first one's, zeroes
+// that one's diagonal and takes the others out of live.  One warp.
+template <int K>
+__device__ __forceinline__ void dense_fold(int32_t *w, int nsv, Mask<K> C, Mask<K> &live) {
+  const int l = threadIdx.x & 31, r = C.first();
+  C.clear(r);
+  int32_t sum[K];
+#pragma unroll
+  for (int j = 0; j < K; ++j) sum[j] = 0;
+  for (Mask<K> c = C; c.any();) {
+    const int x = c.first();
+    c.clear(x);
+#pragma unroll
+    for (int j = 0; j < K; ++j)
+      if (l + 32 * j < nsv) sum[j] += w[x * nsv + l + 32 * j];
+  }
+#pragma unroll
+  for (int j = 0; j < K; ++j) {
+    if (l + 32 * j < nsv) w[r * nsv + l + 32 * j] += sum[j];
+    sum[j] = 0;
+  }
   __syncwarp();
-  if (c < nsv) w[c * nsv + r] += w[c * nsv + l];
+  for (Mask<K> c = C; c.any();) {
+    const int x = c.first();
+    c.clear(x);
+#pragma unroll
+    for (int j = 0; j < K; ++j)
+      if (l + 32 * j < nsv) sum[j] += w[(l + 32 * j) * nsv + x];
+  }
+#pragma unroll
+  for (int j = 0; j < K; ++j) {
+    if (l + 32 * j < nsv) w[(l + 32 * j) * nsv + r] += sum[j];
+    live.w[j] &= ~C.w[j];
+  }
   __syncwarp();
-  if (c == 0) w[r * nsv + r] = 0;
+  if (l == 0) w[r * nsv + r] = 0;
   __syncwarp();
 }
 
-// One maximum-adjacency ordering over the live indices (mask live); kcap > 0
-// caps keys and records merges in duf; kcap == 0 reports s, t and the cut.
-__device__ __forceinline__ void dense_order(const int32_t *w, int nsv, uint32_t live, int kcap,
-                                            int32_t *duf, int &s, int &t, int &cut, bool &merged) {
-  const int l = threadIdx.x & 31;
-  unsigned key = 0;  // at most the item's edges, below 2^30
-  bool added = !((live >> l) & 1u);
-  const int cnt = __popc(live);
-  s = t = -1;
-  cut = 0;
-  merged = false;
-  for (int step = 0; step < cnt; ++step) {
-    // largest key, ties to the smallest index
-    const unsigned top = __reduce_max_sync(FULL, added ? 0u : key);
-    const int X = __ffs(__ballot_sync(FULL, !added && key == top)) - 1;
-    s = t;
-    t = X;
-    cut = (int)top;
-    added |= l == X;
-    const int wx = l < nsv ? w[X * nsv + l] : 0;
-    if (!added && wx > 0) {
-      unsigned nk = key + (unsigned)wx;
-      if (kcap > 0 && nk >= (unsigned)kcap) {
-        nk = (unsigned)kcap;
-        // merge l into X's set (duf links point to smaller indices)
-        volatile int32_t *vd = duf;
-        int a = X, b = l;
-        for (;;) {
-          while (vd[a] != a) a = vd[a];
-          while (vd[b] != b) b = vd[b];
-          if (a == b) break;
-          if (a > b) { const int tt = a; a = b; b = tt; }
-          if (atomicCAS(&duf[b], b, a) == b) break;
-        }
-        merged = true;
-      }
-      key = nk;
-    }
-    __syncwarp();
-  }
-  merged = __any_sync(FULL, merged);
+// The index in left of largest key, ties to the smallest.
+template <int K>
+__device__ __forceinline__ int dense_pick(const unsigned (&key)[K], const Mask<K> &left,
+                                          unsigned &top) {
+  unsigned best = 0u;
+#pragma unroll
+  for (int j = 0; j < K; ++j) best = max(best, left.mine(j) ? key[j] : 0u);
+  top = __reduce_max_sync(FULL, best);
+  Mask<K> m;
+#pragma unroll
+  for (int j = 0; j < K; ++j) m.w[j] = __ballot_sync(FULL, left.mine(j) && key[j] == top);
+  return m.first();
 }
 
 struct DenseResult {
   int cut;        // minimum cut, or -1 when the contraction left one super-vertex
-  uint32_t side;  // the minimum cut's side (mask of initial indices)
+  uint32_t side[DENSE_NSV / 32];  // the minimum cut's side (mask of initial indices)
   int passes, phases;
 };
 
-// Runs the dense finish on w (nsv <= 32 indices; the super-vertices are the
-// indices in live0) with one warp (any warp; all its lanes call).  duf: 32
-// ints of scratch.  Every lane returns the result.
-__device__ __forceinline__ DenseResult dense_finish(int32_t *w, int nsv, uint32_t live0, int kcap, int32_t *duf) {
+// Runs the dense finish on w (nsv <= 32 K indices) with one warp (any warp;
+// all its lanes call).  grp: nsv ints of scratch.  Every lane returns the
+// result (side: K words).
+template <int K>
+__device__ __forceinline__ DenseResult dense_finish(int32_t *w, int nsv, int kcap, int32_t *grp) {
   const int l = threadIdx.x & 31;
-  uint32_t live = live0;
-  uint32_t mem = 1u << l;  // lane l: the initial indices it holds
-  int passes = 0, phases = 0;
-  bool more = true;
-  while (more && __popc(live) > 1) {
-    duf[l] = l;
-    __syncwarp();
-    int s, t, cut;
-    bool merged;
-    dense_order(w, nsv, live, kcap, duf, s, t, cut, merged);
-    ++passes;
-    more = merged;
-    if (!merged) break;
-    // fold every merged index into its root, in ascending order
-    volatile int32_t *vd = duf;
-    for (int x = 0; x < nsv; ++x) {
-      if (!((live >> x) & 1u)) continue;
-      int r = x;
-      while (vd[r] != r) r = vd[r];
-      if (r == x) continue;
-      dense_fold(w, nsv, r, x);
-      const uint32_t mx = __shfl_sync(FULL, mem, x);
-      if (l == r) mem |= mx;
-      live &= ~(1u << x);
-    }
-  }
-  DenseResult res{-1, 0u, passes, 0};
-  while (__popc(live) > 1) {
-    int s, t, cut;
-    bool merged;
-    dense_order(w, nsv, live, 0, duf, s, t, cut, merged);
-    ++phases;
-    if (res.cut < 0 || cut < res.cut) {
-      res.cut = cut;
-      res.side = __shfl_sync(FULL, mem, t);
-    }
-    const int lo = s < t ? s : t, hi = s < t ? t : s;
-    dense_fold(w, nsv, lo, hi);
-    const uint32_t mh = __shfl_sync(FULL, mem, hi);
-    if (l == lo) mem |= mh;
-    live &= ~(1u << hi);
-  }
-  res.phases = phases;
-  __syncwarp();
-  return res;
-}
-
-// The same dense finish for up to DENSE_WIDE_NSV super-vertices: lane l
-// holds indices l, l+32, ... (K per lane); the merged sets are tracked in
-// grp[initial index] = the index that holds it now, and the minimum cut's
-// side is returned as a mask of initial indices (side[j], bit l = index
-// l + 32 j).  Same rules, same results, as dense_finish.
-constexpr int DENSE_WIDE_NSV = 128;
-
-template <int K>
-__device__ __forceinline__ bool dw_live(const uint32_t (&live)[K], int x) {
-  bool r = false;
-#pragma unroll
-  for (int j = 0; j < K; ++j) r = (x >> 5) == j ? ((live[j] >> (x & 31)) & 1u) != 0u : r;
-  return r;
-}
-
-template <int K>
-__device__ __forceinline__ void dw_kill(uint32_t (&live)[K], int x) {
-#pragma unroll
-  for (int j = 0; j < K; ++j)
-    if ((x >> 5) == j) live[j] &= ~(1u << (x & 31));
-}
-
-// Adds row and column x of w into r (r < x), zeroes r's diagonal, moves
-// x's members to r.  One warp.
-template <int K>
-__device__ __forceinline__ void dense_fold_w(int32_t *w, int nsv, int r, int x, int32_t *grp) {
-  const int c = threadIdx.x & 31;
-#pragma unroll
-  for (int j = 0; j < K; ++j) {
-    const int cc = c + 32 * j;
-    if (cc < nsv) w[r * nsv + cc] += w[x * nsv + cc];
-  }
-  __syncwarp();
-#pragma unroll
-  for (int j = 0; j < K; ++j) {
-    const int cc = c + 32 * j;
-    if (cc < nsv) {
-      w[cc * nsv + r] += w[cc * nsv + x];
-      if (grp[cc] == x) grp[cc] = r;
-    }
-  }
-  __syncwarp();
-  if (c == 0) w[r * nsv + r] = 0;
-  __syncwarp();
-}
-
-template <int K>
-__device__ __forceinline__ void dense_order_w(const int32_t *w, int nsv, const uint32_t (&live)[K],
-                                              int kcap, int32_t *duf, int &s, int &t, int &cut,
-                                              bool &merged) {
-  const int l = threadIdx.x & 31;
-  unsigned key[K];  // at most the item's edges, below 2^30
-  bool added[K];
-  int cnt = 0;
-#pragma unroll
-  for (int j = 0; j < K; ++j) {
-    key[j] = 0;
-    added[j] = !((live[j] >> l) & 1u);
-    cnt += __popc(live[j]);
-  }
-  s = t = -1;
-  cut = 0;
-  merged = false;
-  for (int step = 0; step < cnt; ++step) {
-    // largest key, ties to the smallest index
-    unsigned best = 0u;
-#pragma unroll
-    for (int j = 0; j < K; ++j) best = max(best, added[j] ? 0u : key[j]);
-    best = __reduce_max_sync(FULL, best);
-    unsigned first = 0xffffffffu;
-#pragma unroll
-    for (int j = K - 1; j >= 0; --j)
-      if (!added[j] && key[j] == best) first = (unsigned)(l + 32 * j);
-    const int X = (int)__reduce_min_sync(FULL, first);
-    s = t;
-    t = X;
-    cut = (int)best;
-#pragma unroll
-    for (int j = 0; j < K; ++j) {
-      const int idx = l + 32 * j;
-      added[j] |= idx == X;
-      const int wx = idx < nsv ? w[X * nsv + idx] : 0;
-      if (!added[j] && wx > 0) {
-        unsigned nk = key[j] + (unsigned)wx;
-        if (kcap > 0 && nk >= (unsigned)kcap) {
-          nk = (unsigned)kcap;
-          volatile int32_t *vd = duf;
-          int a = X, b = idx;
-          for (;;) {
-            while (vd[a] != a) a = vd[a];
-            while (vd[b] != b) b = vd[b];
-            if (a == b) break;
-            if (a > b) { const int tt = a; a = b; b = tt; }
-            if (atomicCAS(&duf[b], b, a) == b) break;
-          }
-          merged = true;
-        }
-        key[j] = nk;
-      }
-    }
-    __syncwarp();
-  }
-  merged = __any_sync(FULL, merged);
-}
-
-// duf, grp: nsv ints each; side: K words.
-template <int K>
-__device__ __noinline__ DenseResult dense_finish_w(int32_t *w, int nsv, int kcap, int32_t *duf, int32_t *grp,
-                                      uint32_t *side) {
-  const int l = threadIdx.x & 31;
-  uint32_t live[K];
-  int nlive = 0;
+  Mask<K> live;
 #pragma unroll
   for (int j = 0; j < K; ++j) {
     const int b = 32 * j;
-    live[j] = nsv >= b + 32 ? FULL : (nsv > b ? (1u << (nsv - b)) - 1u : 0u);
-    nlive += __popc(live[j]);
+    live.w[j] = nsv >= b + 32 ? FULL : (nsv > b ? (1u << (nsv - b)) - 1u : 0u);
+    // grp[initial index] = the index that holds it now
     if (l + b < nsv) grp[l + b] = l + b;
   }
   __syncwarp();
-  int passes = 0, phases = 0;
-  while (nlive > 1) {
+  DenseResult res;
+  res.cut = -1;
+  res.passes = res.phases = 0;
+#pragma unroll
+  for (int j = 0; j < K; ++j) res.side[j] = 0u;
+  // moves the members of every index in C to its first one
+  auto regroup = [&](const Mask<K> &C) {
+    const int r = C.first();
 #pragma unroll
     for (int j = 0; j < K; ++j)
-      if (l + 32 * j < nsv) duf[l + 32 * j] = l + 32 * j;
-    __syncwarp();
-    int s, t, cut;
-    bool merged;
-    dense_order_w<K>(w, nsv, live, kcap, duf, s, t, cut, merged);
-    ++passes;
-    if (!merged) break;
-    // fold every merged index into its root, in ascending order
-    volatile int32_t *vd = duf;
-    for (int x = 0; x < nsv; ++x) {
-      if (!dw_live<K>(live, x)) continue;
-      int r = x;
-      while (vd[r] != r) r = vd[r];
-      if (r == x) continue;
-      dense_fold_w<K>(w, nsv, r, x, grp);
-      dw_kill<K>(live, x);
-      --nlive;
-    }
-  }
-  DenseResult res{-1, 0u, passes, 0};
-  while (nlive > 1) {
-    int s, t, cut;
-    bool merged;
-    dense_order_w<K>(w, nsv, live, 0, duf, s, t, cut, merged);
-    ++phases;
-    if (res.cut < 0 || cut < res.cut) {
-      res.cut = cut;
+      if (l + 32 * j < nsv) {
+        const int g = grp[l + 32 * j];
+        bool in = false;
 #pragma unroll
-      for (int j = 0; j < K; ++j) {
-        const unsigned b = __ballot_sync(FULL, l + 32 * j < nsv && grp[l + 32 * j] == t);
-        if (l == 0) side[j] = b;
+        for (int i = 0; i < K; ++i) in |= (g >> 5) == i && ((C.w[i] >> (g & 31)) & 1u);
+        if (in) grp[l + 32 * j] = r;
+      }
+  };
+  while (live.count() > 1) {
+    unsigned key[K];
+#pragma unroll
+    for (int j = 0; j < K; ++j) key[j] = 0u;
+    Mask<K> left = live;
+    const Mask<K> start = live;
+    bool merged = false;
+    ++res.passes;
+    // the pass reads the matrix as it was: its phases are folded after it
+    while (left.any()) {
+      unsigned top;
+      const int X = dense_pick<K>(key, left, top);
+      Mask<K> C, todo;
+#pragma unroll
+      for (int j = 0; j < K; ++j) C.w[j] = todo.w[j] = (X >> 5) == j ? 1u << (X & 31) : 0u;
+      left.clear(X);
+      while (todo.any() && left.any()) {
+        const int x = todo.first();
+        todo.clear(x);
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+          if (left.mine(j)) key[j] += (unsigned)w[x * nsv + l + 32 * j];
+          const unsigned sat = __ballot_sync(FULL, left.mine(j) && key[j] >= (unsigned)kcap);
+          C.w[j] |= sat;
+          todo.w[j] |= sat;
+          left.w[j] &= ~sat;
+        }
+      }
+      // members point to their phase's smallest through grp, where only an
+      // index's own entry (grp[x] for live x) is read back below
+      if (C.count() > 1) {
+        merged = true;
+        regroup(C);
+        __syncwarp();
       }
     }
-    const int lo = s < t ? s : t, hi = s < t ? t : s;
-    dense_fold_w<K>(w, nsv, lo, hi, grp);
-    dw_kill<K>(live, hi);
-    --nlive;
+    if (!merged) break;
+    // fold every phase: the live indices by the index that holds them now
+    Mask<K> rest = start;
+    while (rest.any()) {
+      const int r = rest.first();
+      const int g = grp[r];
+      Mask<K> C;
+#pragma unroll
+      for (int j = 0; j < K; ++j) {
+        const bool in = rest.mine(j) && grp[l + 32 * j] == g;
+        C.w[j] = __ballot_sync(FULL, in);
+        rest.w[j] &= ~C.w[j];
+      }
+      if (C.count() > 1) dense_fold<K>(w, nsv, C, live);
+    }
   }
-  res.phases = phases;
+  while (live.count() > 1) {
+    unsigned key[K], cut = 0u;
+#pragma unroll
+    for (int j = 0; j < K; ++j) key[j] = 0u;
+    Mask<K> left = live;
+    int s = -1, t = -1;
+    while (left.any()) {
+      const int X = dense_pick<K>(key, left, cut);
+      s = t;
+      t = X;
+      left.clear(X);
+#pragma unroll
+      for (int j = 0; j < K; ++j)
+        if (left.mine(j)) key[j] += (unsigned)w[X * nsv + l + 32 * j];
+    }
+    ++res.phases;
+    if (res.cut < 0 || (int)cut < res.cut) {
+      res.cut = (int)cut;
+#pragma unroll
+      for (int j = 0; j < K; ++j)
+        res.side[j] = __ballot_sync(FULL, l + 32 * j < nsv && grp[l + 32 * j] == t);
+    }
+    Mask<K> C;
+#pragma unroll
+    for (int j = 0; j < K; ++j)
+      C.w[j] = ((s >> 5) == j ? 1u << (s & 31) : 0u) | ((t >> 5) == j ? 1u << (t & 31) : 0u);
+    regroup(C);
+    __syncwarp();
+    dense_fold<K>(w, nsv, C, live);
+  }
   __syncwarp();
   return res;
 }
 
 // The dense finish of a CTA's item, by its first warp; w: nsv x nsv weights.
 // The result and the cut's side are left in sh for the other warps.
-__device__ __noinline__ void dense_cta(int32_t *w, int nsv, int kcap, Sh *shp) {
-  Sh &sh = *shp;
-  DenseResult dr;
-  if (nsv <= DENSE_NSV) {
-    dr = dense_finish(w, nsv, nsv >= 32 ? 0xffffffffu : (1u << nsv) - 1u, kcap, sh.duf);
-    if (threadIdx.x == 0) sh.wside[0] = dr.side;
-  } else if (nsv <= 64) {
-    dr = dense_finish_w<2>(w, nsv, kcap, sh.wduf, sh.wgrp, sh.wside);
-  } else {
-    dr = dense_finish_w<4>(w, nsv, kcap, sh.wduf, sh.wgrp, sh.wside);
-  }
+template <int K>
+__device__ __forceinline__ void dense_cta_k(int32_t *w, int nsv, int kcap, Sh &sh) {
+  const DenseResult dr = dense_finish<K>(w, nsv, kcap, sh.wgrp);
   if (threadIdx.x == 0) {
+#pragma unroll
+    for (int j = 0; j < K; ++j) sh.wside[j] = dr.side[j];
     sh.dcut = dr.cut;
     sh.dpasses = dr.passes;
     sh.dphases = dr.phases;
   }
+}
+__device__ __noinline__ void dense_cta(int32_t *w, int nsv, int kcap, Sh *shp) {
+  if (nsv <= 32)
+    dense_cta_k<1>(w, nsv, kcap, *shp);
+  else if (nsv <= 64)
+    dense_cta_k<2>(w, nsv, kcap, *shp);
+  else
+    dense_cta_k<4>(w, nsv, kcap, *shp);
 }
 
 // Exact acceptance test for lambda >= kcap by forest certificates.  Take
@@ -1667,7 +1598,7 @@ __device__ __noinline__ int forest_accept(const Mem<IT> *m0, int n, int kcap, in
     nroots = block_sum_int(roots, sh);
     lap(5);
     if (nroots == 1) return round;
-    if (nroots <= DENSE_WIDE_NSV && nroots * nroots <= 2 * (n + 1)) {
+    if (nroots <= DENSE_NSV && nroots * nroots <= 2 * (n + 1)) {
       // few super-vertices: the dense finish's capped passes decide
       int32_t *idx = m.C, *rank = m.H;
       int32_t *w = reinterpret_cast<int32_t *>(m.wide);
@@ -1716,8 +1647,8 @@ struct TinyMask<1> { using T = uint32_t; };
 template <>
 struct TinyMask<2> { using T = unsigned long long; };
 
-// Scratch of one warp, in ints: the weights of at most 32 sets, their
-// union-find, the part stack (32 masks of R words), row bits (32R masks) and
+// Scratch of one warp, in ints: the weights of at most 32 sets, the sets that
+// hold them, the part stack (32 masks of R words), row bits (32R masks) and
 // the degree prefix (32R).
 template <int R>
 __host__ __device__ constexpr size_t tiny_scratch_ints() {
@@ -1785,8 +1716,8 @@ __device__ bool tiny_item_body(const RefineParams &P, unsigned long long seq, co
   const int n = it.n;
   ReqCtx *Rg = &P.reqs[it.req];
   const ReqCtx Rc = load_ctx(Rg);
-  int32_t *w = scratch, *duf = scratch + 32 * 32;
-  M *stk = reinterpret_cast<M *>(duf + 32);
+  int32_t *w = scratch, *grp = scratch + 32 * 32;
+  M *stk = reinterpret_cast<M *>(grp + 32);
   M *rbits = stk + 32;
   int32_t *pre = reinterpret_cast<int32_t *>(rbits + NV);
   int32_t v[R];
@@ -1941,7 +1872,7 @@ __device__ bool tiny_item_body(const RefineParams &P, unsigned long long seq, co
       roots |= C & (~C + 1);
       ++p;
     }
-    DenseResult dr{-1, 0u, 1, 0};
+    int cut = -1, passes = 1, phases = 0;
     M side = 0;
     if (p > 32) return false;  // more sets than the matrix holds: the whole CTA takes the item
     if (p > 1) {
@@ -1970,16 +1901,18 @@ __device__ bool tiny_item_body(const RefineParams &P, unsigned long long seq, co
         }
       }
       __syncwarp();
-      dr = dense_finish(w, p, p >= 32 ? FULL : (1u << p) - 1u, kcap, duf);
-      if (p < nal) ++dr.passes;
+      const DenseResult dr = dense_finish<1>(w, p, kcap, grp);
+      cut = dr.cut;
+      passes = dr.passes + (p < nal ? 1 : 0);
+      phases = dr.phases;
 #pragma unroll
       for (int j = 0; j < R; ++j)
-        side |= (M)__ballot_sync(FULL, mine[j] && ((dr.side >> at[j]) & 1u)) << (32 * j);
+        side |= (M)__ballot_sync(FULL, mine[j] && ((dr.side[0] >> at[j]) & 1u)) << (32 * j);
       __syncwarp();
     }
-    st_passes += dr.passes;
-    st_phases += dr.phases;
-    if (dr.cut < 0) {
+    st_passes += passes;
+    st_phases += phases;
+    if (cut < 0) {
       // accept (Algorithm 3: save V_c); output id resolved after the run
       const int i0 = ffs_m(cur) - 1;
       int32_t minv = __shfl_sync(FULL, v[0], i0 & 31);
@@ -1993,7 +1926,7 @@ __device__ bool tiny_item_body(const RefineParams &P, unsigned long long seq, co
       st_acc += 1;
       continue;
     }
-    if (dr.cut > T) {
+    if (cut > T) {
       failed = true;
       break;
     }
@@ -2470,7 +2403,7 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
       // the weight matrix of the dense finish: in E..F when it fits, else in
       // the dynamic shared memory past what the item occupies
       int32_t *wmat = nullptr;
-      if (nsv <= P.dense_max && nsv <= DENSE_WIDE_NSV) {
+      if (nsv <= P.dense_max && nsv <= DENSE_NSV) {
         if (nsv * nsv <= 2 * (n + 1)) {
           wmat = reinterpret_cast<int32_t *>(m.wide);
         } else {
