@@ -381,9 +381,15 @@ struct Timer {
 };
 
 
-enum RunBuf { R_IN, R_OUT, R_POOL, R_SLOT, R_LMIN, R_RING, R_CTR, R_SLAB, R_REQ, R_INH,
+enum RunBuf { R_IN, R_OUT, R_POOL, R_SLOT, R_LMIN, R_RING, R_CTR, R_SLAB, R_INH,
               R_CM_PARTS, R_CM_PARTOF, R_CM_SCRATCH, R_CM_ITEMS, R_CM_MISC, R_COUNT };
 static_assert(R_COUNT <= 16, "Graph::rb holds 16 buffers");
+
+// What a run reads back at its end, in one copy.
+struct RunEnd {
+  RunCounters ctr;
+  ReqCtx req;
+};
 
 // CM (Section 2.4, Algorithms 4-5): the resolution of its CPM community step.
 struct CmOpts {
@@ -430,11 +436,9 @@ void run_impl(Graph *g, const int32_t *lab_in, const wcc_threshold_rule *rule, i
   auto *lmin = static_cast<int32_t *>(rb[R_LMIN].ensure(4 * n));
   auto *inh = static_cast<unsigned long long *>(rb[R_INH].ensure(8 * n));
   auto *ring = static_cast<QSlot *>(rb[R_RING].ensure(sizeof(QSlot) * cap));
-  auto *ctr = static_cast<RunCounters *>(rb[R_CTR].ensure(sizeof(RunCounters)));
-  auto *req = static_cast<ReqCtx *>(rb[R_REQ].ensure(sizeof(ReqCtx)));
-  WCC_CUDA(cudaMemsetAsync(slot, 0xff, 8 * n, s));
-  WCC_CUDA(cudaMemsetAsync(lmin, 0xff, 4 * n, s));
-  WCC_CUDA(cudaMemsetAsync(ctr, 0, sizeof(RunCounters), s));
+  auto *end = static_cast<RunEnd *>(rb[R_CTR].ensure(sizeof(RunEnd)));
+  RunCounters *ctr = &end->ctr;
+  ReqCtx *req = &end->req;
   ReqCtx hreq{};
   hreq.off = g->off.as<int64_t>();
   hreq.adj = g->adj.as<int32_t>();
@@ -447,9 +451,8 @@ void run_impl(Graph *g, const int32_t *lab_in, const wcc_threshold_rule *rule, i
   hreq.min_size = min_size;
   hreq.rule_num = r.num;
   hreq.rule_den = r.den;
-  WCC_CUDA(cudaMemcpyAsync(req, &hreq, sizeof(hreq), cudaMemcpyHostToDevice, s));
+  run_init(n, slot, lmin, ring, cap, ctr, req, hreq, s);
   if (gi.kept > 0) {
-    WCC_CUDA(cudaMemsetAsync(ring, 0xff, sizeof(QSlot) * cap, s));
     seed_items(gi, n, g->ws, 0, req, pool, slot, ring, cap, ctr, s);
   }
   tm.mark(1, s);
@@ -537,23 +540,17 @@ void run_impl(Graph *g, const int32_t *lab_in, const wcc_threshold_rule *rule, i
   }
   tm.mark(2, s);
   // ---- a9: ids = rank of each accepted cluster's smallest vertex, numbered
-  // into the staging buffer right behind the kernel; the run's counters are
-  // read after it (one wait for both), and the result reaches clustering_out
-  // only once they show no error
-  int32_t *d_out = static_cast<int32_t *>(rb[R_OUT].ensure(4 * n));
-  number_clusters(lmin, n, d_out, g->ws, s);
+  // right behind the kernel; a run that failed writes none of them
+  int32_t *d_out = on_device ? lab_out : static_cast<int32_t *>(rb[R_OUT].ensure(4 * n));
+  number_clusters(lmin, n, d_out, g->ws, s, &ctr->error);
   tm.mark(3, s);
-  RunCounters hc{};
-  ReqCtx hr{};
-  if (gi.kept > 0) {
-    WCC_CUDA(cudaMemcpyAsync(&hc, ctr, sizeof(hc), cudaMemcpyDeviceToHost, s));
-    WCC_CUDA(cudaMemcpyAsync(&hr, req, sizeof(hr), cudaMemcpyDeviceToHost, s));
+  const RunEnd he = read_back(end, s);
+  const ReqCtx &hr = he.req;
+  check_derr(he.ctr.error, "refinement");
+  if (!on_device) {
+    WCC_CUDA(cudaMemcpyAsync(lab_out, d_out, 4 * n, cudaMemcpyDeviceToHost, s));
     WCC_CUDA(cudaStreamSynchronize(s));
-    check_derr(hc.error, "refinement");
   }
-  WCC_CUDA(cudaMemcpyAsync(lab_out, d_out, 4 * n,
-                           on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
-  WCC_CUDA(cudaStreamSynchronize(s));
 
   if (stats) {
     stats->in_clusters = gi.clusters;
@@ -1050,7 +1047,8 @@ int wcc_number_by_minima(const int32_t *minima, int64_t n, int32_t *labels_out, 
       o = static_cast<int32_t *>(dout.ensure(4 * n));
     }
     check_minima(mn, n, ws, s);
-    if (n > 0) number_clusters(mn, n, o, ws, s);
+    unsigned *werr = n > 0 ? number_clusters(mn, n, o, ws, s) : nullptr;
+    if (werr && read_back(werr, s)) check_device_error(DERR_TIMEOUT, "numbering");
     int32_t top = -1;
     if (n > 0) {
       // ids are dense and ascending by smallest vertex: K = 1 + the largest id

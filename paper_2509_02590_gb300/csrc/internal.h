@@ -56,10 +56,10 @@ bool radix_sort_keys_u64(uint64_t *keys, uint64_t *keys_alt, int64_t n, int bits
                          unsigned *err, cudaStream_t s);
 
 // Per-request workspace of the pipeline stages: grown on demand, kept
-// between runs; sk/sv remember where group_by_label() left its sort.
+// between runs; sv remembers where group_by_label() left its sorted vertices.
 struct Workspace {
   DevBuf b[24];
-  uint32_t *sk = nullptr, *sv = nullptr;
+  uint32_t *sv = nullptr;
 };
 
 // ---- csr.cu ----------------------------------------------------------------
@@ -236,8 +236,14 @@ void k_max_i32_launch(const int32_t *a, int64_t n, int32_t *out, cudaStream_t s)
 // WCC_ERR_INVALID unless every entry is -1 or a representative r <= v with
 // minima[r] == r.
 void check_minima(const int32_t *minima, int64_t n, Workspace &ws, cudaStream_t s);
-void number_clusters(const int32_t *label_min, int64_t n, int32_t *out, Workspace &ws,
-                     cudaStream_t s);
+// err (device, NULL: one of its own): nothing is written to out when it is
+// nonzero, and DERR_TIMEOUT is set there when a bounded wait between the
+// numbering's tiles runs out.  Returns the word to check (NULL: none).
+unsigned *number_clusters(const int32_t *label_min, int64_t n, int32_t *out, Workspace &ws,
+                          cudaStream_t s, unsigned *err = nullptr);
+// Slots, cluster minima, ring and counters of a new run, and its context.
+void run_init(int64_t n, unsigned long long *slot, int32_t *lmin, QSlot *ring, uint64_t cap,
+              RunCounters *ctr, ReqCtx *req, const ReqCtx &value, cudaStream_t s);
 
 int64_t bitlen_u64(uint64_t x);
 unsigned grid_for(int64_t n, int per = 256);

@@ -12,8 +12,8 @@ constexpr int TB = 256;
 
 // Workspace slots.
 enum {
-  B_KEYS, B_VALS, B_KEYS2, B_VALS2, B_TEMP, B_HEAD, B_HIDX, B_CSTART, B_PDEG, B_KEEP, B_QIDX,
-  B_DG, B_OK1, B_OV1, B_OK2, B_OV2, B_INFO, B_FLAG, B_RANK, B_BASE, B_COUNT
+  B_KEYS, B_VALS, B_KEYS2, B_VALS2, B_TEMP, B_CL, B_CSTART, B_DSUM, B_KEEP, B_QIDX, B_OK1, B_OV1,
+  B_OK2, B_OV2, B_INFO, B_FLAG, B_RANK, B_BASE, B_COUNT
 };
 static_assert(B_COUNT <= 24, "workspace slots");
 
@@ -25,8 +25,13 @@ struct SeedInfo {
   unsigned err;                 // DERR_* bits
   unsigned maxkey;              // largest label + 1
   unsigned kept;                // clusters with >= min_size members
-  unsigned pad;
+  unsigned ticket;              // tiles handed out (k_clusters)
 };
+
+// Graphs of at most GROUP_SMALL vertices are grouped, seeded and numbered by
+// one CTA each (see k_group_small).
+constexpr int GROUP_SMALL = 8192;
+constexpr int GT = 1024;  // its threads
 
 // keys[v] = label + 1 (0 for unclustered), vals[v] = v; largest key; labels
 // below -1 are malformed.
@@ -45,57 +50,254 @@ __global__ void k_make_keys(const int32_t *__restrict__ lab, int64_t n, uint32_t
   if ((threadIdx.x & 31) == 0 && k) atomicMax(maxkey, k);
 }
 
-__global__ void k_heads(const uint32_t *__restrict__ sk, int64_t n, uint32_t *head) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  head[i] = (sk[i] != 0 && (i == 0 || sk[i - 1] != sk[i])) ? 1u : 0u;
+// ---- single-pass running counts over tiles -----------------------------------
+// A tile's status word: 2 bits of state (its own count, or the count up to its
+// end), 62 of value.  Thread 0 of the tile's block calls; returns the count of
+// all earlier tiles.  Tiles are handed out in order, so every wait ends; one
+// that outlasts a second sets DERR_TIMEOUT.
+constexpr unsigned long long TS_OWN = 1ull << 62, TS_ALL = 2ull << 62, TS_VAL = (1ull << 62) - 1;
+__device__ __forceinline__ unsigned long long tiles_before(unsigned long long *status, int64_t tile,
+                                                           unsigned long long own, unsigned *err) {
+  unsigned long long before = 0;
+  if (tile > 0) {
+    atomicExch(&status[tile], TS_OWN | own);
+    const uint64_t t0 = globaltimer_ns();
+    for (int64_t p = tile - 1; p >= 0;) {
+      const unsigned long long w = *(volatile unsigned long long *)&status[p];
+      if ((w >> 62) == 0) {
+        if (globaltimer_ns() - t0 > 1000ull * 1000 * 1000) {
+          atomicOr(err, DERR_TIMEOUT);
+          break;
+        }
+        continue;
+      }
+      before += w & TS_VAL;
+      if ((w >> 62) == 2ull) break;
+      --p;
+    }
+  }
+  atomicExch(&status[tile], TS_ALL | (before + own));
+  return before;
 }
 
-// cstart[c] = first sorted position of cluster c, cstart[K] = n; also
-// records K and the number of unclustered vertices (they sort first).
-__global__ void k_starts(const uint32_t *__restrict__ head, const uint32_t *__restrict__ hidx,
-                         int64_t n, int64_t *cstart, SeedInfo *info) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t K = hidx[n];
-  if (i < n && head[i]) {
-    cstart[hidx[i]] = i;
-    if (hidx[i] == 0) info->skip = i;
+constexpr int CI = 8;             // sorted positions a thread
+constexpr int CTILE = TB * CI;    // ... and a tile
+
+// The clusters of the sorted labels: cl[i] = the cluster of sorted position i
+// (-1: unclustered), cstart[c] = its first position (cstart[K] = n), dsum[c]
+// += the degrees of its members; also K and the unclustered vertices (they
+// sort first).  One pass: a tile counts its first-of-a-label positions and
+// adds the earlier tiles' count by look-back.
+__global__ void __launch_bounds__(TB) k_clusters(const uint32_t *__restrict__ sk,
+                                                const uint32_t *__restrict__ sv,
+                                                const int64_t *__restrict__ off, int64_t n,
+                                                int32_t *cl, int64_t *cstart,
+                                                unsigned long long *dsum,
+                                                unsigned long long *status, SeedInfo *info) {
+  __shared__ int sm[TB / 32 + 1];
+  __shared__ unsigned tile_sh;
+  __shared__ unsigned long long before_sh;
+  if (threadIdx.x == 0) tile_sh = atomicAdd(&info->ticket, 1u);
+  __syncthreads();
+  const int64_t tile = tile_sh, base = tile * CTILE + (int64_t)threadIdx.x * CI;
+  uint32_t k[CI];
+  long long deg[CI];
+  uint32_t prev = base > 0 && base - 1 < n ? sk[base - 1] : 0u;
+  int heads = 0;
+#pragma unroll
+  for (int z = 0; z < CI; ++z) k[z] = base + z < n ? sk[base + z] : 0u;
+#pragma unroll
+  for (int z = 0; z < CI; ++z) {
+    const uint32_t v = base + z < n && k[z] ? sv[base + z] : 0u;
+    deg[z] = base + z < n && k[z] ? off[v + 1] - off[v] : 0;
   }
-  if (i == 0) {
+  unsigned first = 0u;
+#pragma unroll
+  for (int z = 0; z < CI; ++z) {
+    if (base + z < n && k[z] != 0u && k[z] != prev) {
+      first |= 1u << z;
+      ++heads;
+    }
+    prev = k[z];
+  }
+  int tot;
+  const int ex = block_exclusive_scan<TB>(heads, &tot, sm);
+  if (threadIdx.x == 0) before_sh = tiles_before(status, tile, (unsigned long long)tot, &info->err);
+  __syncthreads();
+  int64_t c = (int64_t)before_sh + ex - 1;  // the cluster the thread's first position continues
+  const int64_t c0 = c + ((first & 1u) ? 1 : 0);
+  const bool whole = first == 0u || first == 1u;  // the thread's positions are one cluster's
+  long long sum = 0;
+#pragma unroll
+  for (int z = 0; z < CI; ++z) {
+    const int64_t i = base + z;
+    if (i >= n) break;
+    if ((first >> z) & 1u) {
+      if (sum) atomicAdd(&dsum[c], (unsigned long long)sum);
+      sum = 0;
+      ++c;
+      cstart[c] = i;
+      if (c == 0) info->skip = i;
+    }
+    cl[i] = k[z] ? (int32_t)c : -1;
+    sum += deg[z];
+  }
+  // the last run's sum, once per warp when the warp is inside one cluster
+  const int64_t lead = __shfl_sync(FULL, c0, 0);
+  const bool same = __all_sync(FULL, whole && c0 == lead);
+  if (same) {
+    sum = warp_sum(sum);
+    if ((threadIdx.x & 31) != 0) sum = 0;
+  }
+  if (sum) atomicAdd(&dsum[c], (unsigned long long)sum);
+  if (threadIdx.x == 0 && tile == (n - 1) / CTILE) {
+    const int64_t K = (int64_t)before_sh + tot;
     cstart[K] = n;
     info->clusters = K;
     if (K == 0) info->skip = n;
   }
 }
 
-// degree of each vertex in sorted order (for the per-cluster degree sums)
-__global__ void k_sorted_deg(const uint32_t *__restrict__ sv, const int64_t *__restrict__ off,
-                             int64_t n, int64_t *dg) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  uint32_t v = sv[i];
-  dg[i] = off[v + 1] - off[v];
-}
-
-__global__ void k_keep(const int64_t *__restrict__ cstart, const uint32_t *__restrict__ Kp,
-                       int64_t cap, int min_size, uint32_t *keep,
-                       const int64_t *__restrict__ pdeg, SeedInfo *info) {
-  int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t K = *Kp;
+// Which clusters are kept, how many, and the largest size and degree sum.
+__global__ void k_keep(const int64_t *__restrict__ cstart, int min_size, uint32_t *keep,
+                       const unsigned long long *__restrict__ dsum, SeedInfo *info) {
+  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t K = info->clusters;
+  if (c - (int64_t)(threadIdx.x & 31) >= K) return;  // the whole warp is past the last cluster
   unsigned long long sz = 0, ds = 0;
-  if (c < cap && c >= K) keep[c] = 0u;
+  bool k = false;
   if (c < K) {
     sz = (unsigned long long)(cstart[c + 1] - cstart[c]);
-    bool k = (int64_t)sz >= min_size;
+    k = (int64_t)sz >= min_size;
     keep[c] = k ? 1u : 0u;
-    if (k) ds = (unsigned long long)(pdeg[cstart[c + 1]] - pdeg[cstart[c]]);
-    else sz = 0;
+    ds = k ? dsum[c] : 0ull;
+    if (!k) sz = 0;
   }
   sz = warp_max(sz);
   ds = warp_max(ds);
+  const unsigned kept = __popc(__ballot_sync(FULL, k));
   if ((threadIdx.x & 31) == 0) {
     if (sz) atomicMax(&info->max_n, sz);
     if (ds) atomicMax(&info->max_dsum, ds);
+    if (kept) atomicAdd(&info->kept, kept);
+  }
+}
+
+// All values a[0..P) ascending, P a power of two, by a block of T threads.
+template <int T>
+__device__ __forceinline__ void block_bitonic(unsigned long long *a, int P) {
+  for (int k = 2; k <= P; k <<= 1)
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      for (int i = threadIdx.x; i < P / 2; i += T) {
+        const int o = i & (j - 1), lo = 2 * (i - o) + o, hi = lo + j;
+        const unsigned long long x = a[lo], y = a[hi];
+        if ((x > y) == ((lo & k) == 0)) {
+          a[lo] = y;
+          a[hi] = x;
+        }
+      }
+      __syncthreads();
+    }
+}
+
+// The whole grouping of a graph of at most GROUP_SMALL vertices by one CTA, in
+// place of about fifteen launches whose gaps would be most of its time: labels
+// sorted with their vertices in shared memory, clusters, degree sums and the
+// queue order as the kernels above and below give them.
+__global__ void __launch_bounds__(GT) k_group_small(const int32_t *__restrict__ lab, int n,
+                                                   const int64_t *__restrict__ off, int min_size,
+                                                   uint32_t *sv, int32_t *cl, int64_t *cstart,
+                                                   uint32_t *keep, uint32_t *qidx, SeedInfo *info) {
+  extern __shared__ __align__(16) unsigned long long a[];
+  __shared__ int sm[GT / 32 + 1];
+  __shared__ unsigned bad, kept;
+  __shared__ int skip;
+  __shared__ unsigned long long max_n, max_d;
+  if (threadIdx.x == 0) {
+    bad = kept = 0u;
+    skip = n;
+    max_n = max_d = 0ull;
+  }
+  __syncthreads();
+  int P = 2;
+  while (P < n) P <<= 1;
+  for (int i = threadIdx.x; i < P; i += GT) {
+    unsigned long long key = ~0ull;
+    if (i < n) {
+      const int32_t c = lab[i];
+      if (c < -1) bad = 1u;
+      key = ((unsigned long long)(unsigned)(c + 1) << 32) | (unsigned)i;
+    }
+    a[i] = key;
+  }
+  __syncthreads();
+  if (bad) {
+    if (threadIdx.x == 0) {
+      SeedInfo r{};
+      r.err = DERR_INVALID;
+      *info = r;
+    }
+    return;
+  }
+  block_bitonic<GT>(a, P);
+  int K = 0;
+  for (int i0 = 0; i0 < n; i0 += GT) {
+    const int i = i0 + threadIdx.x;
+    const unsigned key = i < n ? (unsigned)(a[i] >> 32) : 0u;
+    const bool head = key != 0u && (i == 0 || (unsigned)(a[i - 1] >> 32) != key);
+    int tot;
+    const int ex = block_exclusive_scan<GT>(head ? 1 : 0, &tot, sm);
+    if (i < n) {
+      const int c = K + ex + (head ? 1 : 0) - 1;
+      sv[i] = (unsigned)a[i];
+      cl[i] = key ? c : -1;
+      if (head) cstart[c] = i;
+      if (head && c == 0) skip = i;
+    }
+    K += tot;
+  }
+  if (threadIdx.x == 0) cstart[K] = n;
+  __syncthreads();
+  for (int c = threadIdx.x; c < K; c += GT) a[c] = 0ull;  // degree sums
+  __syncthreads();
+  for (int i = threadIdx.x; i < n; i += GT) {
+    const int c = cl[i];
+    const uint32_t v = sv[i];
+    if (c >= 0) atomicAdd(&a[c], (unsigned long long)(off[v + 1] - off[v]));
+  }
+  __syncthreads();
+  for (int c = threadIdx.x; c < K; c += GT) {
+    const unsigned long long sz = (unsigned long long)(cstart[c + 1] - cstart[c]);
+    const bool k = (int64_t)sz >= min_size;
+    keep[c] = k ? 1u : 0u;
+    if (k) {
+      atomicAdd(&kept, 1u);
+      atomicMax(&max_n, sz);
+      atomicMax(&max_d, a[c]);
+    }
+  }
+  __syncthreads();
+  // queue order: kept clusters first, larger ones earlier
+  int Q = 2;
+  while (Q < K) Q <<= 1;
+  for (int c = threadIdx.x; c < Q; c += GT) {
+    unsigned long long key = ~0ull;
+    if (c < K)
+      key = ((keep[c] ? max_n - (unsigned long long)(cstart[c + 1] - cstart[c]) : max_n + 1) << 32) |
+            (unsigned)c;
+    a[c] = key;
+  }
+  __syncthreads();
+  block_bitonic<GT>(a, Q);
+  for (int i = threadIdx.x; i < (int)kept; i += GT) qidx[(unsigned)a[i]] = (uint32_t)i;
+  if (threadIdx.x == 0) {
+    SeedInfo r{};
+    r.max_n = max_n;
+    r.max_dsum = max_d;
+    r.clusters = K;
+    r.skip = skip;
+    r.kept = kept;
+    *info = r;
   }
 }
 
@@ -132,20 +334,7 @@ __global__ void __launch_bounds__(1024) k_order_small(const int64_t *__restrict_
     a[i] = v;
   }
   __syncthreads();
-  for (int k = 2; k <= P; k <<= 1)
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int i = threadIdx.x; i < P; i += blockDim.x) {
-        const int l = i ^ j;
-        if (l > i) {
-          const unsigned long long x = a[i], y = a[l];
-          if ((x > y) == ((i & k) == 0)) {
-            a[i] = y;
-            a[l] = x;
-          }
-        }
-      }
-      __syncthreads();
-    }
+  block_bitonic<1024>(a, P);
   for (int i = threadIdx.x; i < nkept; i += blockDim.x) qidx[(uint32_t)a[i]] = (uint32_t)i;
 }
 
@@ -156,63 +345,159 @@ __global__ void k_invert(const uint32_t *__restrict__ order, int64_t nkept, uint
 
 // Reserves queue indices [base, base + nkept) for the items of one request
 // and counts them as pending (globally and for the request) before any of
-// them is published.
+// them is published.  One thread.
+__device__ __forceinline__ unsigned long long reserve(RunCounters *ctr, ReqCtx *ctx,
+                                                      long long nkept) {
+  atomicAdd(reinterpret_cast<unsigned long long *>(&ctx->pending),
+            static_cast<unsigned long long>(nkept));
+  atomicAdd(reinterpret_cast<unsigned long long *>(&ctr->pending),
+            static_cast<unsigned long long>(nkept));
+  __threadfence();
+  const unsigned long long b = atomicAdd(&ctr->tail, (unsigned long long)nkept);
+  ctx->seed_end = b + (unsigned long long)nkept;
+  return b;
+}
 __global__ void k_reserve(RunCounters *ctr, ReqCtx *ctx, long long nkept,
                           unsigned long long *base) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    atomicAdd(reinterpret_cast<unsigned long long *>(&ctx->pending),
-              static_cast<unsigned long long>(nkept));
-    atomicAdd(reinterpret_cast<unsigned long long *>(&ctr->pending),
-              static_cast<unsigned long long>(nkept));
-    __threadfence();
-    const unsigned long long b = atomicAdd(&ctr->tail, (unsigned long long)nkept);
-    *base = b;
-    ctx->seed_end = b + (unsigned long long)nkept;
-  }
+  if (threadIdx.x == 0 && blockIdx.x == 0) *base = reserve(ctr, ctx, nkept);
 }
+
+// What seeding reads: the grouping's arrays.
+struct SeedIn {
+  const uint32_t *sv;
+  const int32_t *cl;
+  const int64_t *cstart;
+  const uint32_t *keep, *qidx;
+  int64_t n, skip, K;
+};
 
 // pool[i - skip] = sorted vertex; slot[v] = (queue index << 32) | rank
-__global__ void k_pool_slots(const uint32_t *__restrict__ sv, const uint32_t *__restrict__ head,
-                             const uint32_t *__restrict__ hidx, const int64_t *__restrict__ cstart,
-                             const uint32_t *__restrict__ keep, const uint32_t *__restrict__ qidx,
-                             const unsigned long long *__restrict__ base, int64_t n, int64_t skip,
-                             int32_t *pool, unsigned long long *slot) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n || i < skip) return;
-  uint32_t v = sv[i];
-  pool[i - skip] = (int32_t)v;
-  int64_t c = (int64_t)hidx[i] + head[i] - 1;  // inclusive head count - 1
-  if (keep[c])
-    slot[v] = ((unsigned long long)queue_tag(*base + qidx[c]) << 32) | (unsigned)(i - cstart[c]);
+__device__ __forceinline__ void seed_vertex(const SeedIn &in, int64_t i, unsigned long long base,
+                                            int32_t *pool, unsigned long long *slot) {
+  const uint32_t v = in.sv[i];
+  pool[i - in.skip] = (int32_t)v;
+  const int32_t c = in.cl[i];
+  if (in.keep[c])
+    slot[v] = ((unsigned long long)queue_tag(base + in.qidx[c]) << 32) |
+              (unsigned)(i - in.cstart[c]);
 }
 
-// Descriptors of the kept clusters, then their publication.
-__global__ void k_seed(const int64_t *__restrict__ cstart, const uint32_t *__restrict__ keep,
-                       const uint32_t *__restrict__ qidx, const unsigned long long *__restrict__ base,
-                       int64_t K, int64_t skip, uint16_t req, QSlot *ring, uint64_t cap) {
-  int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= K || !keep[c]) return;
-  uint64_t q = *base + qidx[c];
+// The descriptor of a kept cluster, then its publication.
+__device__ __forceinline__ void seed_cluster(const SeedIn &in, int64_t c, unsigned long long base,
+                                             uint16_t req, QSlot *ring, uint64_t cap) {
+  const uint64_t q = base + in.qidx[c];
   QSlot *s = &ring[q % cap];
-  s->item.vbeg = cstart[c] - skip;
-  s->item.n = (int32_t)(cstart[c + 1] - cstart[c]);
+  s->item.vbeg = in.cstart[c] - in.skip;
+  s->item.n = (int32_t)(in.cstart[c + 1] - in.cstart[c]);
   s->item.flags = ITEM_TOP;
   s->item.req = req;
   __threadfence();
   atomicExch((unsigned long long *)&s->seq, (unsigned long long)q);
 }
 
-__global__ void k_out_flags(const int32_t *__restrict__ lmin, int64_t n, uint32_t *flag) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) flag[i] = lmin[i] == (int32_t)i ? 1u : 0u;
+__global__ void k_pool_slots(SeedIn in, const unsigned long long *__restrict__ base, int32_t *pool,
+                             unsigned long long *slot) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < in.n && i >= in.skip) seed_vertex(in, i, *base, pool, slot);
+}
+
+__global__ void k_seed(SeedIn in, const unsigned long long *__restrict__ base, uint16_t req,
+                       QSlot *ring, uint64_t cap) {
+  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (c < in.K && in.keep[c]) seed_cluster(in, c, *base, req, ring, cap);
+}
+
+// The three steps above in one launch, for a small graph.
+__global__ void __launch_bounds__(GT) k_seed_small(SeedIn in, RunCounters *ctr, ReqCtx *ctx,
+                                                  long long nkept, uint16_t req, int32_t *pool,
+                                                  unsigned long long *slot, QSlot *ring,
+                                                  uint64_t cap) {
+  __shared__ unsigned long long base;
+  if (threadIdx.x == 0) base = reserve(ctr, ctx, nkept);
+  __syncthreads();
+  for (int64_t i = in.skip + threadIdx.x; i < in.n; i += GT) seed_vertex(in, i, base, pool, slot);
+  __threadfence();
+  __syncthreads();
+  for (int64_t c = threadIdx.x; c < in.K; c += GT)
+    if (in.keep[c]) seed_cluster(in, c, base, req, ring, cap);
+}
+
+// rank[v] = representatives (label_min[v] == v) before v, in one pass over
+// tiles (see tiles_before).
+__global__ void __launch_bounds__(TB) k_rank(const int32_t *__restrict__ lmin, int64_t n,
+                                            uint32_t *rank, unsigned long long *status,
+                                            unsigned *ticket, unsigned *err) {
+  __shared__ int sm[TB / 32 + 1];
+  __shared__ unsigned tile_sh;
+  __shared__ unsigned long long before_sh;
+  if (threadIdx.x == 0) tile_sh = atomicAdd(ticket, 1u);
+  __syncthreads();
+  const int64_t tile = tile_sh, base = tile * CTILE + (int64_t)threadIdx.x * CI;
+  int32_t l[CI];
+#pragma unroll
+  for (int z = 0; z < CI; ++z) l[z] = base + z < n ? lmin[base + z] : -1;
+  int mine = 0;
+#pragma unroll
+  for (int z = 0; z < CI; ++z) mine += base + z < n && l[z] == (int32_t)(base + z);
+  int tot;
+  const int ex = block_exclusive_scan<TB>(mine, &tot, sm);
+  if (threadIdx.x == 0) before_sh = tiles_before(status, tile, (unsigned long long)tot, err);
+  __syncthreads();
+  uint32_t r = (uint32_t)before_sh + (uint32_t)ex;
+#pragma unroll
+  for (int z = 0; z < CI; ++z) {
+    if (base + z >= n) break;
+    rank[base + z] = r;
+    r += l[z] == (int32_t)(base + z);
+  }
+}
+
+// Both steps of the numbering for a small graph, by one CTA.
+__global__ void __launch_bounds__(GT) k_number_small(const int32_t *__restrict__ lmin, int n,
+                                                    int32_t *out, const unsigned *err) {
+  extern __shared__ __align__(16) unsigned long long a[];
+  int32_t *rank = reinterpret_cast<int32_t *>(a);
+  __shared__ int sm[GT / 32 + 1];
+  if (err && *err) return;
+  int carry = 0;
+  for (int i0 = 0; i0 < n; i0 += GT) {
+    const int i = i0 + threadIdx.x;
+    const int f = i < n && lmin[i] == i ? 1 : 0;
+    int tot;
+    const int ex = block_exclusive_scan<GT>(f, &tot, sm);
+    if (i < n) rank[i] = carry + ex;
+    carry += tot;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < n; i += GT) {
+    const int32_t r = lmin[i];
+    out[i] = r >= 0 ? rank[r] : -1;
+  }
 }
 
 __global__ void k_out_final(const int32_t *__restrict__ lmin, const uint32_t *__restrict__ rank,
-                            int64_t n, int32_t *out) {
+                            int64_t n, int32_t *out, const unsigned *err) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+  if (i >= n || *err) return;
   int32_t r = lmin[i];
   out[i] = r >= 0 ? (int32_t)rank[r] : -1;
+}
+
+// The state a run starts from: every vertex in no item and no cluster, no ring
+// slot published, the counters zero, the request's context.
+__global__ void k_run_init(int64_t n, unsigned long long *slot, int32_t *lmin, QSlot *ring,
+                           uint64_t cap, RunCounters *ctr, ReqCtx *req, ReqCtx value) {
+  const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = i0; i < n; i += step) {
+    slot[i] = ~0ull;
+    lmin[i] = -1;
+  }
+  for (int64_t i = i0; i < (int64_t)cap; i += step) ring[i].seq = ~0ull;
+  if (i0 == 0) {
+    *ctr = RunCounters{};
+    *req = value;
+  }
 }
 
 template <typename T>
@@ -250,11 +535,45 @@ GroupInfo group_by_label(const int64_t *off, int64_t n, const int32_t *labels, i
   GroupInfo gi{};
   uint32_t *keys = buf<uint32_t>(ws, B_KEYS, n);
   uint32_t *vals = buf<uint32_t>(ws, B_VALS, n);
+  int32_t *cl = buf<int32_t>(ws, B_CL, n);
+  int64_t *cstart = buf<int64_t>(ws, B_CSTART, n + 1);
+  uint32_t *keep = buf<uint32_t>(ws, B_KEEP, n + 1);
+  uint32_t *qidx = buf<uint32_t>(ws, B_QIDX, n + 1);
+  auto fill = [&](const SeedInfo &hi) {
+    if (hi.err) check_device_error(hi.err, "grouping");
+    gi.clusters = hi.clusters;
+    gi.skip = hi.skip;
+    gi.kept = (int64_t)hi.kept;
+    gi.max_n = (int64_t)hi.max_n;
+    gi.max_dsum = (int64_t)hi.max_dsum;
+  };
+  if (n <= GROUP_SMALL) {
+    SeedInfo *info = buf<SeedInfo>(ws, B_INFO, 1);
+    size_t P = 2;
+    while ((int64_t)P < n) P <<= 1;
+    if (8 * P > 32 * 1024)
+      WCC_CUDA(cudaFuncSetAttribute(k_group_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    8 * GROUP_SMALL));
+    k_group_small<<<1, GT, 8 * P, s>>>(labels, (int)n, off, min_size, vals, cl, cstart, keep, qidx,
+                                       info);
+    note_launch();
+    WCC_CUDA(cudaGetLastError());
+    const SeedInfo hi = read_back(info, s);
+    if (hi.err) check_device_error(hi.err, "clustering_in");
+    ws.sv = vals;
+    fill(hi);
+    return gi;
+  }
   uint32_t *keys2 = buf<uint32_t>(ws, B_KEYS2, n);
   uint32_t *vals2 = buf<uint32_t>(ws, B_VALS2, n);
   void *temp = ws.b[B_TEMP].ensure(std::max(radix_temp_bytes(n), scan_temp_bytes(n + 1)));
-  SeedInfo *info = buf<SeedInfo>(ws, B_INFO, 1);
-  WCC_CUDA(cudaMemsetAsync(info, 0, sizeof(SeedInfo), s));
+  // the counters, the tiles' status words and the degree sums start at zero
+  const int64_t tiles = (n + CTILE - 1) / CTILE;
+  const size_t zero = sizeof(SeedInfo) + 8 * (size_t)tiles + 8 * (size_t)n;
+  SeedInfo *info = static_cast<SeedInfo *>(ws.b[B_INFO].ensure(zero));
+  unsigned long long *status = reinterpret_cast<unsigned long long *>(info + 1);
+  unsigned long long *dsum = status + tiles;
+  WCC_CUDA(cudaMemsetAsync(info, 0, zero, s));
   k_make_keys<<<grid_for(n), TB, 0, s>>>(labels, n, keys, vals, &info->maxkey, &info->err);
   note_launch();
   WCC_CUDA(cudaGetLastError());
@@ -266,43 +585,19 @@ GroupInfo group_by_label(const int64_t *off, int64_t n, const int32_t *labels, i
     sk = keys2;
     sv = vals2;
   }
-  ws.sk = sk;
   ws.sv = sv;
-  uint32_t *head = buf<uint32_t>(ws, B_HEAD, n + 1);
-  uint32_t *hidx = buf<uint32_t>(ws, B_HIDX, n + 1);
-  k_heads<<<grid_for(n), TB, 0, s>>>(sk, n, head); note_launch();
-  WCC_CUDA(cudaGetLastError());
-  // hidx[n] receives the number of distinct labels K; arrays indexed by
-  // cluster are sized by n so that K need not be read back here
-  exclusive_scan_u32(head, hidx, n, hidx + n, temp, s);
-  int64_t *cstart = buf<int64_t>(ws, B_CSTART, n + 1);
-  k_starts<<<grid_for(n), TB, 0, s>>>(head, hidx, n, cstart, info); note_launch();
-  // per-cluster degree sums (prefix sums of degrees in sorted order)
-  int64_t *dg = buf<int64_t>(ws, B_DG, n + 1);
-  int64_t *pdeg = buf<int64_t>(ws, B_PDEG, n + 1);
-  uint32_t *keep = buf<uint32_t>(ws, B_KEEP, n + 1);
-  uint32_t *qidx = buf<uint32_t>(ws, B_QIDX, n + 1);
-  k_sorted_deg<<<grid_for(n), TB, 0, s>>>(sv, off, n, dg); note_launch();
-  WCC_CUDA(cudaMemsetAsync(dg + n, 0, 8, s));
-  exclusive_scan_i64(dg, pdeg, n + 1, nullptr, temp, s);
-  k_keep<<<grid_for(n), TB, 0, s>>>(cstart, hidx + n, n, min_size, keep, pdeg, info);
+  k_clusters<<<(unsigned)tiles, TB, 0, s>>>(sk, sv, off, n, cl, cstart, dsum, status, info);
   note_launch();
-  exclusive_scan_u32(keep, qidx, n, &info->kept, temp, s);
+  k_keep<<<grid_for(n), TB, 0, s>>>(cstart, min_size, keep, dsum, info); note_launch();
   WCC_CUDA(cudaGetLastError());
-  SeedInfo hi = read_back(info, s);
-  if (hi.err) check_device_error(hi.err, "grouping");
-  gi.clusters = hi.clusters;
-  gi.skip = hi.skip;
-  gi.kept = (int64_t)hi.kept;
-  gi.max_n = (int64_t)hi.max_n;
-  gi.max_dsum = (int64_t)hi.max_dsum;
+  fill(read_back(info, s));
   const int64_t K = gi.clusters;
-  if (gi.kept > 1 && K <= ORDER_SMALL) {
+  if (gi.kept > 0 && K <= ORDER_SMALL) {
     // queue order: largest input clusters first (qidx = rank by size), in one block
     k_order_small<<<1, 1024, 0, s>>>(cstart, keep, K, (uint32_t)gi.max_n, gi.kept, qidx);
     note_launch();
     WCC_CUDA(cudaGetLastError());
-  } else if (gi.kept > 1) {
+  } else if (gi.kept > 0) {
     // queue order: largest input clusters first (qidx = rank by size)
     uint32_t *ok1 = buf<uint32_t>(ws, B_OK1, K);
     uint32_t *ov1 = buf<uint32_t>(ws, B_OV1, K);
@@ -326,20 +621,24 @@ void seed_items(const GroupInfo &gi, int64_t n, Workspace &ws, uint16_t req, Req
                 int32_t *pool, unsigned long long *slot, QSlot *ring, uint64_t cap,
                 RunCounters *ctr, cudaStream_t s) {
   if (gi.kept <= 0) return;
+  const SeedIn in{ws.sv,
+                  static_cast<int32_t *>(ws.b[B_CL].p),
+                  static_cast<int64_t *>(ws.b[B_CSTART].p),
+                  static_cast<uint32_t *>(ws.b[B_KEEP].p),
+                  static_cast<uint32_t *>(ws.b[B_QIDX].p),
+                  n,
+                  gi.skip,
+                  gi.clusters};
+  if (n <= GROUP_SMALL) {
+    k_seed_small<<<1, GT, 0, s>>>(in, ctr, ctx_dev, gi.kept, req, pool, slot, ring, cap);
+    note_launch();
+    WCC_CUDA(cudaGetLastError());
+    return;
+  }
   unsigned long long *base = buf<unsigned long long>(ws, B_BASE, 1);
   k_reserve<<<1, 32, 0, s>>>(ctr, ctx_dev, gi.kept, base); note_launch();
-  k_pool_slots<<<grid_for(n), TB, 0, s>>>(ws.sv, static_cast<uint32_t *>(ws.b[B_HEAD].p),
-                                          static_cast<uint32_t *>(ws.b[B_HIDX].p),
-                                          static_cast<int64_t *>(ws.b[B_CSTART].p),
-                                          static_cast<uint32_t *>(ws.b[B_KEEP].p),
-                                          static_cast<uint32_t *>(ws.b[B_QIDX].p), base, n,
-                                          gi.skip, pool, slot);
-  note_launch();
-  k_seed<<<grid_for(gi.clusters), TB, 0, s>>>(static_cast<int64_t *>(ws.b[B_CSTART].p),
-                                              static_cast<uint32_t *>(ws.b[B_KEEP].p),
-                                              static_cast<uint32_t *>(ws.b[B_QIDX].p), base,
-                                              gi.clusters, gi.skip, req, ring, cap);
-  note_launch();
+  k_pool_slots<<<grid_for(n), TB, 0, s>>>(in, base, pool, slot); note_launch();
+  k_seed<<<grid_for(gi.clusters), TB, 0, s>>>(in, base, req, ring, cap); note_launch();
   WCC_CUDA(cudaGetLastError());
 }
 
@@ -426,15 +725,33 @@ void check_minima(const int32_t *minima, int64_t n, Workspace &ws, cudaStream_t 
   if (h) fail(WCC_ERR_INVALID, "minima: an entry is not the smallest vertex of a cluster");
 }
 
-void number_clusters(const int32_t *label_min, int64_t n, int32_t *out, Workspace &ws,
-                     cudaStream_t s) {
-  uint32_t *flag = buf<uint32_t>(ws, B_FLAG, n);
-  uint32_t *rank = buf<uint32_t>(ws, B_RANK, n);
-  void *temp = ws.b[B_TEMP].ensure(std::max(radix_temp_bytes(n), scan_temp_bytes(n + 1)));
-  k_out_flags<<<grid_for(n), TB, 0, s>>>(label_min, n, flag); note_launch();
-  exclusive_scan_u32(flag, rank, n, nullptr, temp, s);
-  k_out_final<<<grid_for(n), TB, 0, s>>>(label_min, rank, n, out); note_launch();
+void run_init(int64_t n, unsigned long long *slot, int32_t *lmin, QSlot *ring, uint64_t cap,
+              RunCounters *ctr, ReqCtx *req, const ReqCtx &value, cudaStream_t s) {
+  const int64_t most = std::max<int64_t>(n, (int64_t)cap);
+  k_run_init<<<std::min<unsigned>(grid_for(most), 152 * 16), TB, 0, s>>>(n, slot, lmin, ring, cap,
+                                                                       ctr, req, value);
+  note_launch();
   WCC_CUDA(cudaGetLastError());
+}
+
+unsigned *number_clusters(const int32_t *label_min, int64_t n, int32_t *out, Workspace &ws,
+                          cudaStream_t s, unsigned *err) {
+  if (n <= GROUP_SMALL) {
+    k_number_small<<<1, GT, 4 * (size_t)n, s>>>(label_min, (int)n, out, err); note_launch();
+    WCC_CUDA(cudaGetLastError());
+    return nullptr;
+  }
+  uint32_t *rank = buf<uint32_t>(ws, B_RANK, n);
+  const int64_t tiles = (n + CTILE - 1) / CTILE;
+  const size_t zero = 8 * (size_t)(tiles + 1);
+  unsigned long long *status = static_cast<unsigned long long *>(ws.b[B_FLAG].ensure(zero));
+  unsigned *ticket = reinterpret_cast<unsigned *>(status + tiles);
+  if (!err) err = ticket + 1;
+  WCC_CUDA(cudaMemsetAsync(status, 0, zero, s));
+  k_rank<<<(unsigned)tiles, TB, 0, s>>>(label_min, n, rank, status, ticket, err); note_launch();
+  k_out_final<<<grid_for(n), TB, 0, s>>>(label_min, rank, n, out, err); note_launch();
+  WCC_CUDA(cudaGetLastError());
+  return err;
 }
 
 }  // namespace wccg

@@ -154,10 +154,14 @@ void free_slot(Server *S, Request *R) {
 void finalize(Server *S, Request *R) {
   try {
     ReqCtx *ctx = S->reqtab.as<ReqCtx>() + R->slot;
-    number_clusters(R->lmin.as<int32_t>(), R->n, R->d_out.as<int32_t>(), R->ws, S->astream);
+    unsigned *derr = number_clusters(R->lmin.as<int32_t>(), R->n, R->d_out.as<int32_t>(), R->ws,
+                                     S->astream);
+    unsigned herr = 0;
+    if (derr) WCC_CUDA(cudaMemcpyAsync(&herr, derr, 4, cudaMemcpyDeviceToHost, S->astream));
     WCC_CUDA(cudaMemcpyAsync(R->h_out.data(), R->d_out.p, 4 * R->n, cudaMemcpyDeviceToHost,
                              S->astream));
     ReqCtx h = read_back(ctx, S->astream);
+    if (herr) check_device_error(DERR_TIMEOUT, "numbering");
     R->stats.in_clusters = R->gi.clusters;
     R->stats.out_clusters = h.accepted;
     R->stats.items = h.items;

@@ -1,0 +1,61 @@
+"""Grouping, seeding and numbering at the sizes where they change form: one CTA
+up to 8,192 vertices, tiles of 2,048 sorted positions above, the queue order by
+one block up to 4,096 clusters.  The refinement's result must be the oracle's."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _labels(kind, n, rng):
+    if kind == "none":
+        return np.full(n, -1, np.int32)
+    if kind == "one":
+        return np.full(n, 2**31 - 1, np.int32)
+    if kind == "distinct":
+        return rng.permutation(n).astype(np.int32)
+    if kind == "pairs":  # n // 2 clusters: around the one-block order's limit
+        return (rng.permutation(n) // 2).astype(np.int32)
+    lab = rng.integers(0, max(1, n // 40), n).astype(np.int32)  # "mixed": some unclustered
+    lab[rng.random(n) < 0.2] = -1
+    return lab
+
+
+@pytest.mark.parametrize("n", [1, 2, 33, 1023, 1024, 1025, 8191, 8192, 8193, 10_239, 10_240, 10_241])
+@pytest.mark.parametrize("kind", ["none", "one", "distinct", "pairs", "mixed"])
+def test_sizes(n, kind):
+    import paper_2509_02590_gb300 as wcc
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    rng = np.random.default_rng(n)
+    lab = _labels(kind, n, rng)
+    m = min(3 * n, 6000 if kind == "one" else 3 * n)
+    u, v = rng.integers(0, n, m), rng.integers(0, n, m)
+    same = np.nonzero(lab >= 0)[0]
+    if kind in ("pairs", "mixed") and len(same):  # edges inside the clusters
+        order = same[np.argsort(lab[same], kind="stable")]
+        u, v = np.concatenate([u, order[:-1]]), np.concatenate([v, order[1:]])
+    src, dst = synth.graphs._dedup(n, u, v)
+    off, adj = oracle.build_csr(n, src, dst)
+    ref, _ = oracle.wcc(n, off, adj, lab, 2)
+    with wcc.WccGraph.from_edges(src, dst, n) as g:
+        dev = g.run(torch.from_numpy(lab).cuda(), min_size=2).cpu().numpy()
+        host, st = g.run(lab, min_size=2, stats=True)
+    assert np.array_equal(dev, ref) and np.array_equal(host, ref)
+    assert st["in_clusters"] == len(np.unique(lab[lab >= 0]))
+
+
+@pytest.mark.parametrize("n", [100, 9000])
+def test_labels_below_minus_one_are_refused(n):
+    import paper_2509_02590_gb300 as wcc
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    lab = np.zeros(n, np.int32)
+    lab[n // 2] = -2
+    with wcc.WccGraph.from_edges(np.array([0], np.int32), np.array([1], np.int32), n) as g:
+        with pytest.raises(wcc.WccError):
+            g.run(lab)
