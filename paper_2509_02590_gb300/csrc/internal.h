@@ -214,7 +214,8 @@ struct GroupInfo {
 // a2: groups the vertices of labels (device) by input label (stable radix
 // sort), computes the kept clusters, their sizes and degree sums, and orders
 // them largest first.  Leaves its arrays in ws for seed_items().  One
-// read-back inside (the sort width) plus one at the end (the result).
+// read-back at the end (the result); above the one-CTA limit, one before the
+// sort too (its width).
 GroupInfo group_by_label(const int64_t *off, int64_t n, const int32_t *labels, int min_size,
                          Workspace &ws, cudaStream_t s);
 

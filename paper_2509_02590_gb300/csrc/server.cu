@@ -96,8 +96,9 @@ size_t estimate_bytes(int64_t n) { return (size_t)n * 240 + (1u << 20); }
 size_t graph_bytes(int64_t n, int64_t m) { return 2 * (8 * (size_t)(n + 1) + 8 * (size_t)m); }
 
 // The builder's transient memory while one such graph is built (the edge
-// copies, two 64-bit key arrays and two 32-bit flag arrays over the 2m
-// directed entries, scan and sort temporaries), rounded up: needed only
+// copies and, by buckets, one 64-bit and one 32-bit entry array over the 2m
+// directed entries; by the radix sort, two 64-bit key arrays, two 32-bit flag
+// arrays, scan and sort temporaries: the larger), rounded up: needed only
 // during the admission that builds it.
 size_t build_bytes(int64_t n, int64_t m) { return 2 * (56 * (size_t)m + 8 * (size_t)n) + (1u << 20); }
 
