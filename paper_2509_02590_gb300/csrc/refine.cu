@@ -2625,7 +2625,8 @@ __device__ __forceinline__ bool fetch_item(const RefineParams &P, unsigned long 
 // tail), by compare-and-swap, and then waits -- bounded by wait_limit_ns --
 // for its publication.  With nothing reserved it waits for more: the kernel
 // ends when nothing is pending and the queue is closed, or (open, serving)
-// once one CTA has found nothing pending for idle_limit_ns and set closing;
+// once one CTA has found nothing pending for idle_limit_ns and set closing
+// (what is queued by then waits for the next launch);
 // a wait for work that is pending but never published ends at wait_limit_ns
 // with DERR_TIMEOUT.
 __global__ void __launch_bounds__(RB, 1) k_refine(RefineParams P) {
@@ -2692,6 +2693,13 @@ __global__ void __launch_bounds__(RB, 1) k_refine(RefineParams P) {
           // queue keeps everything not yet claimed).  A CTA takes one item
           // before it looks, so that every step makes progress.
           if (P.stop_flag && took && *P.stop_flag) break;
+          // an open (serving) kernel leaves as a whole: the first CTA that
+          // idled out closes it for all, and the host relaunches it for what
+          // was admitted meanwhile.  Looked at before the queue: work that
+          // arrives while the CTAs are leaving would otherwise run on the few
+          // that found it, and under load those never see the queue empty
+          // (a stream of 1,318 requests/s then completes 184/s).
+          if (vctr->closing) break;
           const unsigned long long h = vctr->head, t = vctr->tail;
           if (h < t) {
             if (atomicCAS(&ctr->head, h, h + 1) == h) {
@@ -2703,11 +2711,6 @@ __global__ void __launch_bounds__(RB, 1) k_refine(RefineParams P) {
             continue;
           }
           if (P.stop_flag && *P.stop_flag) break;
-          // an open (serving) kernel leaves as a whole: the first CTA that
-          // idled out closes it for all, so that work admitted meanwhile
-          // never runs on a few stragglers; the host relaunches it for that
-          // work
-          if (vctr->closing) break;
           const long long pend = vctr->pending;
           const uint64_t waited = globaltimer_ns() - t0;
           if (pend <= 0) {
