@@ -97,8 +97,7 @@ struct Item {
                   // ITEM_INH: a side of a cut split whose parent left first-pass records
   uint16_t req;   // request it belongs to (index into the request table)
 };
-                  // ITEM_VOID: the index of a part that the CTA which split it off refines itself
-enum : uint16_t { ITEM_TOP = 1u, ITEM_INH = 2u, ITEM_VOID = 4u };
+enum : uint16_t { ITEM_TOP = 1u, ITEM_INH = 2u };
 
 // One refinement request: its graph, its per-vertex state and its counters.
 // wcc_run uses one; a server keeps a table of them for the requests it has

@@ -178,7 +178,6 @@ struct Sh {
   int32_t ncta;                // items for the whole CTA
   int32_t has_own;             // the CTA keeps a part of its last item as its next one
   Item own;
-  unsigned long long own_seq;
   Item cta_item[TINY_BLOCK + 1];
   unsigned long long cta_seq[TINY_BLOCK + 1];
   unsigned long long tst[7];   // statistics of the batch's small items
@@ -411,6 +410,13 @@ __device__ __noinline__ int components_af(const Mem<IT> *m0, int64_t d, int n, S
 // that are published fill the front of the range.  Returns that child's tag
 // (-1: none) and, in *emitted, the members published ahead of it.
 //
+// With keep_own, that child is written to the pool like the others but not
+// published: the CTA takes it as its next item (sh.own) under the queue index
+// seq of the item it came from, which no one else uses any more.  A queue
+// index then always stands for an unclaimed item, so that a request's
+// unclaimed indices stay at half its vertices; the price is that a member of
+// the parent which is in no child must not keep the parent's tag in its slot.
+//
 // This and the other parts of an item that are rare, long or used at several
 // places are not inlined (item_mem says how they find the item's memory): the
 // kernel's code then fits the instruction cache better and its main path the
@@ -421,7 +427,7 @@ __device__ __noinline__ int emit_children(const RefineParams &P, const ReqCtx &R
                                           uint16_t req, const Mem<IT> *m0, int64_t d, int which,
                                           int n, int64_t vbeg, Sh *shp, uint16_t cflags = 0,
                                           bool keep_largest = false, int *emitted = nullptr,
-                                          bool keep_own = false) {
+                                          bool keep_own = false, unsigned long long seq = 0ull) {
   Sh &sh = *shp;
   const Mem<IT> m = item_mem<IT, SM>(m0, n, d);
   const int32_t *tag = which == TAG_H ? m.H : m.B;
@@ -443,10 +449,10 @@ __device__ __noinline__ int emit_children(const RefineParams &P, const ReqCtx &R
     __syncthreads();
   }
   const int big = sh.u1 ? 0x7fffffff - (int)(unsigned)(sh.u1 & 0xffffffffull) : -1;
-  const int L = keep_own ? -1 : big;
+  const int L = keep_own ? -1 : big, own = keep_own ? big : -1;
   for (int t = threadIdx.x; t < n; t += RB) {
     bool keep = cnt[t] >= R.min_size && t != L;
-    cidx[t] = keep ? 1 : 0;
+    cidx[t] = keep && t != own ? 1 : 0;
     cbase[t] = keep ? cnt[t] : 0;
     run[t] = 0;
   }
@@ -454,14 +460,23 @@ __device__ __noinline__ int emit_children(const RefineParams &P, const ReqCtx &R
   int nchild = block_scan_array(cidx, n, sh);
   const int total = block_scan_array(cbase, n, sh);
   if (emitted) *emitted = total;
-  if (nchild == 0) return L;
+  if (nchild == 0 && own < 0) return L;
   if (threadIdx.x == 0) {
-    // a kept part and its void index are pending both
-    const long long pend = (long long)nchild + (keep_own ? 1 : 0);
+    const long long pend = (long long)nchild + (own >= 0 ? 1 : 0);
     add_ll(&Rg->pending, pend);
     add_ll(&P.ctr->pending, pend);
     __threadfence();
-    sh.u0 = atomicAdd(&P.ctr->tail, (unsigned long long)nchild);
+    sh.u0 = nchild > 0 ? atomicAdd(&P.ctr->tail, (unsigned long long)nchild) : 0ull;
+  }
+  if (own >= 0) {
+    // members in no child: a side that is too small, or no longer alive (of
+    // those, the ones an earlier split published have another item's tag)
+    for (int i = threadIdx.x; i < n; i += RB) {
+      const int t = tag[i];
+      if (t >= 0 && cnt[t] >= R.min_size) continue;
+      unsigned long long *sl = &R.slot[m.gid[i]];
+      if (t >= 0 || (uint32_t)(__ldcg(sl) >> 32) == queue_tag(seq)) *sl = ~0ull;
+    }
   }
   __syncthreads();
   const unsigned long long s0 = sh.u0;
@@ -481,7 +496,7 @@ __device__ __noinline__ int emit_children(const RefineParams &P, const ReqCtx &R
         int pos = before + rank;
         int32_t v = m.gid[i];
         R.pool[vbeg + cbase[t] + pos] = v;
-        R.slot[v] = ((unsigned long long)queue_tag(s0 + cidx[t]) << 32) | (unsigned)pos;
+        R.slot[v] = ((unsigned long long)queue_tag(t == own ? seq : s0 + cidx[t]) << 32) | (unsigned)pos;
         if (rank == 0) run[t] = before + __popc(peers);
       }
       __syncwarp();
@@ -492,22 +507,18 @@ __device__ __noinline__ int emit_children(const RefineParams &P, const ReqCtx &R
   // descriptors, then publication
   for (int t = threadIdx.x; t < n; t += RB) {
     if (cnt[t] < R.min_size || t == L) continue;
-    unsigned long long q = s0 + cidx[t];
-    QSlot *sl = &P.ring[q % P.ring_cap];
     const Item child{vbeg + cbase[t], cnt[t], cflags, req};
-    if (keep_own && t == big) {
+    if (t == own) {
       sh.own = child;
-      sh.own_seq = q;
       sh.has_own = 1;
-      sl->item = Item{0, 0, ITEM_VOID, req};
     } else {
-      sl->item = child;
+      P.ring[(s0 + cidx[t]) % P.ring_cap].item = child;
     }
   }
   __threadfence();
   __syncthreads();
   for (int t = threadIdx.x; t < n; t += RB) {
-    if (cnt[t] < R.min_size || t == L) continue;
+    if (cnt[t] < R.min_size || t == L || t == own) continue;
     unsigned long long q = s0 + cidx[t];
     atomicExch((unsigned long long *)&P.ring[q % P.ring_cap].seq, q);
   }
@@ -2556,7 +2567,7 @@ __device__ __noinline__ int process_item(const RefineParams &P, unsigned long lo
     // vertices 38.7 -> 37.2 ms a step, small clusters 2M 3.98 -> 3.77)
     emit_children<IT, SM>(P, R, Rg, it.req, &m, dbound, TAG_B, n, vb, &sh,
                           inh_valid ? ITEM_INH : (uint16_t)0, false, nullptr,
-                          P.stop_flag == nullptr && !P.single_item);
+                          P.stop_flag == nullptr && !P.single_item, seq);
   return OUT_CUT_SPLIT;
 }
 
@@ -2773,13 +2784,6 @@ __global__ void __launch_bounds__(RB, 1) k_refine(RefineParams P) {
       pc = t;
     }
     if (!sh.go) break;
-    if (sh.first.flags & ITEM_VOID) {
-      // the index of a kept part counts as pending of its own, so that a
-      // request holds its queue indices until all of them are claimed
-      if (threadIdx.x == 0) finish_items(P, sh.first.req, 1);
-      __syncthreads();  // read by all before the next claim
-      continue;
-    }
     if (tiny_ok && sh.first.n <= tiny_lim) {
       // every warp takes the batch's items one after the other
       const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, k = sh.claim_k;
@@ -2837,10 +2841,10 @@ __global__ void __launch_bounds__(RB, 1) k_refine(RefineParams P) {
     }
     const int ncta = sh.ncta;
     for (int k = 0; k < ncta;) {
-      // the part kept from the last item, else the next of the batch
-      const bool own = sh.has_own != 0;
-      const Item it = own ? sh.own : sh.cta_item[k];
-      const unsigned long long iseq = own ? sh.own_seq : sh.cta_seq[k];
+      // the part kept from the last item (under its index), else the next of
+      // the batch
+      const Item it = sh.has_own ? sh.own : sh.cta_item[k];
+      const unsigned long long iseq = sh.cta_seq[k];
       __syncthreads();
       if (threadIdx.x == 0) sh.has_own = 0;
       if (P.prof && threadIdx.x == 0) {

@@ -252,3 +252,31 @@ def test_serving_submit_does_not_wait_for_the_device(wcc):
     assert max(times) < busy_ms / 2, (times, busy_ms)
     for out in outs:
         assert np.array_equal(out, ref_small)
+
+
+def test_serving_queue_bound_with_clusters_of_many_cuts(wcc):
+    """Clusters that are cut dozens of times (chains of 33 bridged triangles:
+    30 cuts each), almost as many as the queue of a small budget admits.  The
+    parts wait behind all input clusters, so the queue holds most of them at
+    once; each waiting part needs one index for at least two vertices, which is
+    what a request reserves.  With a second index a cut the 1,850 clusters
+    refined before the last is claimed would need 111,000 of the queue's
+    102,400."""
+    tri, count = 33, 2000
+    size, t = 3 * tri, 3 * np.arange(tri)
+    eu = np.concatenate([t, t, t + 1, t[:-1] + 2])
+    ev = np.concatenate([t + 1, t + 2, t + 2, t[1:]])
+    base = size * np.arange(count)[:, None]
+    n = size * count
+    perm = np.random.default_rng(0).permutation(n)
+    src, dst = perm[(base + eu).ravel()].astype(np.int32), perm[(base + ev).ravel()].astype(np.int32)
+    labels = np.empty(n, np.int32)
+    labels[perm] = np.arange(n) // size
+    off, adj = oracle.build_csr(n, src, dst)
+    with wcc.WccGraph.from_edges(src, dst, n) as g, wcc.WccServer(200 << 20) as srv:
+        for min_size in (2, 4):  # 4: the triangles cut off are dropped
+            ref, st = oracle.wcc(n, off, adj, labels, min_size)
+            out, got = srv.wait(srv.submit(g, labels, min_size=min_size), timeout_ms=120_000)
+            assert np.array_equal(out, ref)
+            assert got["splits"] == 30 * count == st["splits"]
+            assert np.array_equal(g.run(labels, min_size=min_size), ref)
