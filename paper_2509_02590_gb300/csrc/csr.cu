@@ -69,7 +69,7 @@ constexpr size_t SMALL_SMEM = 4 * (size_t)(2 * SMALL_ROWS + 1 + SMALL_ENTRIES);
 
 // What a build reports back in one copy.
 struct Result {
-  unsigned err, big, over;  // DERR_* bits, large buckets, a part too long
+  unsigned err, big, over;  // DERR_* bits, large buckets, a bucket or part too long
   uint32_t placed;          // entries in the buckets (the loops' excluded)
   int64_t nnz;
 };
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(1024) k_starts1(Plan p, const uint32_t *__rest
   }
   if (d == 0) start[p.nhigh] = tot;
   if (p.low == 0) return;
-  const uint32_t t = (c + TILE - 1) / TILE;
+  const uint32_t t = c / TILE + (c % TILE != 0u);  // (c + TILE - 1 can wrap)
   const uint32_t t0 = block_exclusive_scan<1024>(t, &tot, sm);
   if (d < (int)p.nhigh) {
     tile0[d] = t0;
@@ -436,14 +436,20 @@ __global__ void __launch_bounds__(SB) k_bucket_sort(Plan p, const uint32_t *__re
   __shared__ int32_t scan[SB / 32 + 1];
   __shared__ int nlong;
   const uint32_t q = blockIdx.x, base = start[q];
-  const int size = (int)(start[q + 1] - base);
+  const uint32_t entries = start[q + 1] - base;  // up to 2^32 - 2, with many copies of an edge
   const int64_t row0 = (int64_t)q << p.s;
   const int rows = (int)min((int64_t)1 << p.s, p.n - row0);
   if (threadIdx.x == 0 && q == p.nb - 1) res->placed = start[p.nb];
-  if (size > BUCKET_CAP) {
-    if (threadIdx.x == 0) big[atomicAdd(&res->big, 1u)] = q;
+  if (entries > (uint32_t)BUCKET_CAP) {
+    if (threadIdx.x == 0) {
+      if (entries > (uint32_t)INT32_MAX)
+        res->over = 1u;
+      else
+        big[atomicAdd(&res->big, 1u)] = q;
+    }
     return;
   }
+  const int size = (int)entries;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int r = threadIdx.x; r < SUB_MAX; r += SB) cnt[r] = 0;
   if (threadIdx.x == 0) nlong = 0;

@@ -84,3 +84,33 @@ def test_builder_refuses_endpoints_out_of_range(n, m, bad):
     u[m // 2] = n if bad == "n" else bad
     with pytest.raises(wcc.WccError):
         wcc.WccGraph.from_edges(u.astype(np.int32), v.astype(np.int32), n)
+
+
+def _copies_of_one_edge(extra):
+    """2^30 + extra edges on 900,000 vertices, all but 5,000 of them 0-1: more
+    than 2^31 entries in the first bucket, which holds rows 0 and 1.  Run in a
+    process of its own, whose device memory (about 130 GB) goes with it."""
+    import paper_2509_02590_gb300 as wcc
+    n, m, k = 900_000, 2**30 + extra, 5000
+    u, v = _random(n, k, 30)
+    src = torch.zeros(m, dtype=torch.int32, device="cuda")
+    dst = torch.ones(m, dtype=torch.int32, device="cuda")
+    src[7:7 + k] = torch.from_numpy(u.astype(np.int32)).cuda()
+    dst[7:7 + k] = torch.from_numpy(v.astype(np.int32)).cuda()
+    off, adj = oracle.build_csr(n, np.append(u, 0).astype(np.int32), np.append(v, 1).astype(np.int32))
+    with wcc.WccGraph.from_edges(src, dst, n) as g:
+        goff, gadj = g.csr()
+    assert np.array_equal(goff, off) and np.array_equal(gadj, adj)
+
+
+def test_bucket_of_more_than_2_31_entries():
+    import os
+    import subprocess
+    import sys
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    if torch.cuda.mem_get_info()[0] < 160 << 30:
+        pytest.skip("needs 160 GB of free device memory")
+    code = "import tests.test_gpu_csr_buckets as t; t._copies_of_one_edge(10_000)"
+    subprocess.run([sys.executable, "-c", code], check=True, timeout=300,
+                   cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
