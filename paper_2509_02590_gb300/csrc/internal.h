@@ -134,6 +134,7 @@ struct RunCounters {
   unsigned int err_info;       // first failing detail (debug aid)
   int open;                    // 1 while a server may still add work (kernel idles instead of exiting)
   int closing;                 // set by the first CTA of an open kernel that idled out: all leave
+  unsigned long long kept_ns;  // %globaltimer when a CTA last kept a part of its own item
 };
 
 // Optional per-item profile record (phase durations in SM cycles: load,

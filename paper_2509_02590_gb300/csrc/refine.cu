@@ -467,6 +467,7 @@ __device__ __noinline__ int emit_children(const RefineParams &P, const ReqCtx &R
     add_ll(&P.ctr->pending, pend);
     __threadfence();
     sh.u0 = nchild > 0 ? atomicAdd(&P.ctr->tail, (unsigned long long)nchild) : 0ull;
+    if (own >= 0) atomicMax(&P.ctr->kept_ns, (unsigned long long)globaltimer_ns());
   }
   if (own >= 0) {
     // members in no child: a side that is too small, or no longer alive (of
@@ -2601,6 +2602,15 @@ __device__ int run_item(const RefineParams &P, unsigned long long seq, const Ite
                 : process_item<int32_t, false>(P, seq, it, slab, dsum, sh);
 }
 
+// Whether a wait for work that began at t0 has outlasted the limit.  A CTA
+// that goes on with a part of its own item may publish nothing for long: the
+// time counts from the last part kept so, as it would from a published one.
+__device__ __forceinline__ bool outlasted(const volatile RunCounters *c, uint64_t t0,
+                                          uint64_t limit_ns) {
+  return globaltimer_ns() - t0 > limit_ns &&
+         (long long)(globaltimer_ns() - c->kept_ns) > (long long)limit_ns;
+}
+
 // Waits (bounded) for queue index q to be published and reads its item
 // with two 8-byte loads.  False, with DERR_TIMEOUT set, when the wait runs
 // out or the run has failed meanwhile.
@@ -2678,7 +2688,7 @@ __global__ void __launch_bounds__(RB, 1) k_refine(RefineParams P) {
             break;
           }
           if (vctr->pending <= 0) break;
-          if (globaltimer_ns() - t0 > P.wait_limit_ns) {
+          if (outlasted(vctr, t0, P.wait_limit_ns)) {
             atomicOr(&ctr->error, DERR_TIMEOUT);
             break;
           }
@@ -2730,7 +2740,7 @@ __global__ void __launch_bounds__(RB, 1) k_refine(RefineParams P) {
               atomicExch(&ctr->closing, 1);
               break;
             }
-          } else if (waited > P.wait_limit_ns) {
+          } else if (outlasted(vctr, t0, P.wait_limit_ns)) {
             atomicOr(&ctr->error, DERR_TIMEOUT);
             break;
           }

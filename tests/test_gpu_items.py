@@ -200,3 +200,26 @@ def test_bounded_queue_wait_times_out_then_recovers(wcc, monkeypatch):
         assert np.array_equal(out.cpu().numpy(), ref)
         out = g.run(lab, min_size=w.min_size, mode="plain")
         assert np.array_equal(out.cpu().numpy(), ref)
+
+
+def test_a_chain_of_kept_parts_counts_as_work(wcc, monkeypatch):
+    """A ring of 160 cliques of 10, cut one clique after the other, the cliques
+    below min_size: the CTA goes on with the rest each time and publishes
+    nothing, for longer than the wait limit in all, while a single cut takes
+    far less.  The idle CTAs wait on."""
+    k, b = 10, 160
+    iu, ju = np.triu_indices(k, 1)
+    base = k * np.arange(b)[:, None]
+    eu = np.concatenate([(base + iu).ravel(), base.ravel() + 1])
+    ev = np.concatenate([(base + ju).ravel(), (base.ravel() + k) % (b * k)])
+    w = _finish(np.random.default_rng(2), b * k, eu, ev, [0] * (b * k), 11, "clique ring")
+    off, adj = oracle.build_csr(w.n, w.src, w.dst)
+    ref, st = oracle.wcc(w.n, off, adj, w.labels, w.min_size)
+    assert st["splits"] > 100
+    with wcc.WccGraph.from_edges(w.src, w.dst, w.n) as g:
+        out, full = g.run(w.labels, min_size=w.min_size, stats=True)
+        assert np.array_equal(out, ref)
+        limit = int(full["ms_refine"] / 4)
+        assert limit >= 10  # the longest cut, the first, takes about 1/50 of the run
+        monkeypatch.setenv("WCC_WAIT_LIMIT_MS", str(limit))
+        assert np.array_equal(g.run(w.labels, min_size=w.min_size), ref)
