@@ -2901,8 +2901,12 @@ __global__ void __launch_bounds__(RB, 1) k_refine(RefineParams P) {
           for (int z = 0; z < 6; ++z) q->fdbg[z] = sh.fdbg[z];
         }
       }
-      if (threadIdx.x == 0) finish_items(P, it.req, 1);
+      if (threadIdx.x == 0) {
+        finish_items(P, it.req, 1);
+        sh.go = vctr->error == 0;
+      }
       __syncthreads();
+      if (!sh.go) break;  // the run has failed: a chain of kept parts ends too
       if (P.prof && threadIdx.x == 0) {
         const long long t = clock64();
         cp.cta += t - pc;

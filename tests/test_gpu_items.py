@@ -223,3 +223,37 @@ def test_a_chain_of_kept_parts_counts_as_work(wcc, monkeypatch):
         assert limit >= 10  # the longest cut, the first, takes about 1/50 of the run
         monkeypatch.setenv("WCC_WAIT_LIMIT_MS", str(limit))
         assert np.array_equal(g.run(w.labels, min_size=w.min_size), ref)
+
+
+def _clique_ring(b):
+    """A ring of b cliques of 10, in one cluster: with min_size 11 it is cut b - 1
+    times, one clique falling off each time."""
+    k = 10
+    iu, ju = np.triu_indices(k, 1)
+    base = k * np.arange(b)[:, None]
+    eu = np.concatenate([(base + iu).ravel(), base.ravel() + 1])
+    ev = np.concatenate([(base + ju).ravel(), (base.ravel() + k) % (b * k)])
+    return _finish(np.random.default_rng(2), b * k, eu, ev, [0] * (b * k), 11, "clique ring")
+
+
+def test_a_failed_run_ends_between_kept_parts(wcc, monkeypatch):
+    """The idle CTAs' wait runs out while one CTA works through a chain of parts
+    it keeps: the run ends after the part in hand, not after the chain, and the
+    next run gives the oracle's result."""
+    import time
+    w = _clique_ring(160)
+    off, adj = oracle.build_csr(w.n, w.src, w.dst)
+    ref, _ = oracle.wcc(w.n, off, adj, w.labels, w.min_size)
+    with wcc.WccGraph.from_edges(w.src, w.dst, w.n) as g:
+        g.run(w.labels, min_size=w.min_size)
+        t0 = time.perf_counter()
+        assert np.array_equal(g.run(w.labels, min_size=w.min_size), ref)
+        full = time.perf_counter() - t0
+        monkeypatch.setenv("WCC_WAIT_LIMIT_MS", "1")
+        t0 = time.perf_counter()
+        with pytest.raises(wcc.WccError) as e:
+            g.run(w.labels, min_size=w.min_size)
+        assert e.value.status == -4  # WCC_ERR_TIMEOUT
+        assert time.perf_counter() - t0 < full / 4
+        monkeypatch.delenv("WCC_WAIT_LIMIT_MS")
+        assert np.array_equal(g.run(w.labels, min_size=w.min_size), ref)
