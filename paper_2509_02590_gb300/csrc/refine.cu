@@ -54,6 +54,15 @@ extern __shared__ __align__(16) char wcc_dyn_smem[];
 // Components that a contraction pass finds one after the other; beyond that
 // many the union-find finds all at once.
 constexpr int MAX_COMP = 32;
+// A search for components alone (CCR) that has added fewer than THIN_FRONT
+// vertices a round on average, after THIN_ROUNDS of them, leaves the item to the
+// union-find too: a round costs about 1,000 cycles whatever it adds, the
+// union-find about 30 ns a vertex whatever the diameter.  One path of 50,000
+// vertices 29.7 -> 2.7 ms, 200 of 2,000 1.66 -> 0.38, 200 chains of 300 triangles
+// 0.94 -> 0.30 (after 16 or 64 rounds: 0.28, 0.35); without the average a 300 x 300
+// grid takes 4.8 ms instead of 2.4.
+constexpr int THIN_ROUNDS = 32;
+constexpr int THIN_FRONT = 32;
 // Rows of more entries are extracted by all warps together.
 constexpr int LONG_ROW = 1024;
 // Most small input clusters a CTA claims at once (see k_refine).  With one per
@@ -850,16 +859,17 @@ __device__ __forceinline__ void warp_push4(const bool (&take)[4], const int (&v)
 // vertex of key 0 starts another component (every vertex of the one before
 // has been added); with more than one, H[i] = the smallest member of i's
 // component, -1 if dead; past MAX_COMP the pass gives up (-2).  With kcap = 1
-// the phases are the components.  Uses C, D, F, G, H and the keys.  Keys are
+// the phases are the components; a pass run for them alone (ccr: rep is B)
+// gives up on long thin items too.  Uses C, D, F, G, H and the keys.  Keys are
 // 16 bits (an increment past kcap is possible while several threads hit one
 // vertex, at most one per thread, so a half-word never overflows into the
 // other).
 template <typename IT, bool SM>
-__device__ __noinline__ int2 first_pass(const Mem<IT> *m0, int64_t d, bool rep_in_b, int n, int nalive,
+__device__ __noinline__ int2 first_pass(const Mem<IT> *m0, int64_t d, bool ccr, int n, int nalive,
                                         int kcap, unsigned *err, Sh *shp) {
   Sh &sh = *shp;
   const Mem<IT> m = item_mem<IT, SM>(m0, n, d);
-  int32_t *rep = rep_in_b ? m.B : m.A;
+  int32_t *rep = ccr ? m.B : m.A;
   uint32_t *kw = m.kw;
   volatile uint16_t *kh = reinterpret_cast<volatile uint16_t *>(m.kw);
   int32_t *queue = m.D, *phmin = m.C, *lr = m.G;
@@ -922,6 +932,7 @@ __device__ __noinline__ int2 first_pass(const Mem<IT> *m0, int64_t d, bool rep_i
     int head = tail++;
     __syncthreads();
     while (head < tail && tail < nalive) {
+      if (ccr && rounds >= THIN_ROUNDS && tail < THIN_FRONT * rounds) return make_int2(-2, 0);
       const int F = tail - head, U = nalive - tail;
       int32_t *qn = &sh.qn[r];
       const int rn = r == 2 ? 0 : r + 1;

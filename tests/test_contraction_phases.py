@@ -121,3 +121,41 @@ def test_refinement_at_loop_edges(monkeypatch, rule, env):
             out, st = g.run(w.labels, min_size=w.min_size, rule=rule, stats=True)
         assert np.array_equal(out, ref), (turn, rule, env)
         assert st["out_clusters"] == int(ref.max(initial=-1)) + 1
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("env", [{}, {"WCC_TINY_N": "0", "WCC_SMEM_KB": "16"}])
+def test_components_of_long_thin_clusters(monkeypatch, env):
+    """Clusters of paths, whose components take as many rounds to grow as the
+    paths are long: around the rounds after which the union-find takes over, in
+    one path and summed over several, and far beyond; after a star of 1,100
+    leaves, which a round adds at once, only after as many more.  With T = 0 the
+    components are the output."""
+    torch = pytest.importorskip("torch")
+    import paper_2509_02590_gb300 as wcc
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    for k, v in env.items():
+        monkeypatch.setenv(k, v)
+    clusters = [[L] for L in (32, 33, 34, 35, 64, 65, 66, 67, 129, 1000, 5000)]
+    clusters += [[33, 33], [33, 34], [17, 17, 17], [2, 65], [65, 2], [3, 2000, 1], [2] * 40]
+    clusters += [[-1100, L] for L in (30, 34, 35, 36, 70)]  # -k: a star of k leaves
+    for shuffled in (False, True):
+        eu, ev, lab, base = [], [], [], 0
+        for c, paths in enumerate(clusters):
+            for L in paths:
+                size = L if L > 0 else 1 - L
+                eu.append(base + (np.arange(L - 1) if L > 0 else np.zeros(-L, np.int64)))
+                ev.append(base + np.arange(1, size))
+                lab.append(np.full(size, c))
+                base += size
+        perm = np.random.default_rng(1).permutation(base) if shuffled else np.arange(base)
+        s, d = synth.graphs._dedup(base, perm[np.concatenate(eu)], perm[np.concatenate(ev)])
+        labels = np.empty(base, np.int32)
+        labels[perm] = np.concatenate(lab)
+        off, adj = oracle.build_csr(base, s, d)
+        ref, _ = oracle.wcc(base, off, adj, labels, 2, kind=oracle.RULE_LINEAR, num=0, den=1)
+        assert ref.max() + 1 == sum(abs(L) > 1 for paths in clusters for L in paths)
+        with wcc.WccGraph.from_edges(s, d, base) as g:
+            out = g.run(labels, min_size=2, rule="linear", num=0, den=1)
+        assert np.array_equal(out, ref)
