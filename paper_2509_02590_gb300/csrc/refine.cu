@@ -177,6 +177,8 @@ struct Sh {
   long long pf_forest_cycles, pf_t0;
   long long fdbg[6];
   int32_t qn[3];                  // contraction pass: super-vertices pushed in a round
+  int32_t ngrp;                   // ... groups touched since the last pick
+  int32_t grp_all;                // ... or all of them
   unsigned long long wbest[RW];   // contraction pass: each warp's best unadded key
   Item first;         // the claimed item
   unsigned long long first_seq;
@@ -757,6 +759,20 @@ constexpr int KEY_MAX = 0x3fff;         // largest kcap the 16-bit keys hold
 // often within its first 32 entries.
 constexpr int PULL_MIN = 64;
 constexpr int PULL_STEP = 32;
+// Picks of an item with 32-bit local ids (65,535 vertices or more) go by groups
+// of 64 vertices, each with its best key: after the usual small round only the
+// groups of the vertices it touched are looked through again (after at most
+// PICK_ROUNDS rounds of at most RW rows of at most PICK_ROW entries, else all).
+// With all keys looked through for every pick the passes of one random cluster
+// of mean degree 12 grow with the square of its size: whole runs at 66,000 /
+// 200,000 / 500,000 vertices take 81 / 1,285 / 7,149 ms, by groups 42 / 287 / 869.
+// Below 65,535 vertices the keys are in shared memory and a look at all of them
+// is at most 64 words a thread.
+constexpr int PICK_GROUP = 64;
+constexpr int PICK_ROUNDS = 8;
+constexpr int PICK_ROW = 256;
+static_assert(PICK_ROUNDS * RW * PICK_ROW + PICK_ROUNDS + 1 <= 65535 - 65535 / PICK_GROUP,
+              "a phase's touched groups fit the array beside the groups' best keys");
 
 // The entries of up to 32 rows, lane r holding row r = adj[b .. b + d), walked
 // by one warp as one flat range.  Calls fn(j, base) for every 128 entries:
@@ -883,8 +899,16 @@ __device__ __noinline__ int2 first_pass(const Mem<IT> *m0, int64_t d, bool ccr, 
   }
   for (int i = threadIdx.x; i < n; i += RB) rep[i] = -1;
   if (threadIdx.x < 3) sh.qn[threadIdx.x] = 0;
-  if (threadIdx.x == 0) sh.ntouched = 0;
+  if (threadIdx.x == 0) sh.ntouched = sh.ngrp = sh.grp_all = 0;
   int tail = 0, phases = 0, r = 0, rounds = 0, comps = 0, comp = -1;
+  // 32-bit local ids: every group's best key ((key << 6 | 63 - place) + 1, 0:
+  // none), then the list of groups touched since the last pick
+  constexpr bool GROUPS = sizeof(IT) == 4;
+  const int ng = (n + PICK_GROUP - 1) / PICK_GROUP;
+  unsigned *gbest = reinterpret_cast<unsigned *>(m.H);
+  int32_t *glist = m.H + ng;
+  bool gall = true;  // all groups are to be looked through
+  int marked = 0;    // rounds since the last pick
   __syncthreads();
   while (tail < nalive) {
     // the phase's first vertex: largest key, then smallest id
@@ -902,13 +926,41 @@ __device__ __noinline__ int2 first_pass(const Mem<IT> *m0, int64_t d, bool ccr, 
       X = best ? (int)(0xffffu - (best & 0xffffu)) : -1;
       fresh = (best >> 16) == 0u;
     } else {
-      unsigned long long best = 0ull;
-      for (int w = threadIdx.x; w < nw; w += RB) {
-        const uint32_t k2 = kw[w];
+      gall = gall || sh.grp_all != 0;
+      auto look = [&](int g, uint32_t k2) {  // group g's best key from its words, one a lane
         const unsigned lo = k2 & 0xffffu, hi = k2 >> 16;
-        const unsigned long long id = ~(unsigned)(2 * w);
-        if (lo < (unsigned)kcap) best = max(best, ((unsigned long long)lo << 32) | id);
-        if (hi < (unsigned)kcap) best = max(best, ((unsigned long long)hi << 32) | (id - 1));
+        unsigned b = lo < (unsigned)kcap ? ((lo << 6) | (unsigned)(63 - 2 * lane)) + 1u : 0u;
+        if (hi < (unsigned)kcap) b = max(b, ((hi << 6) | (unsigned)(62 - 2 * lane)) + 1u);
+        b = __reduce_max_sync(FULL, b);
+        if (lane == 0) gbest[g] = b;
+      };
+      auto words = [&](int g) {  // (no key below kcap past the end)
+        const int w = g * (PICK_GROUP / 2) + lane;
+        return w < nw ? kw[w] : FULL;
+      };
+      if (gall) {
+        for (int g0 = warp; g0 < ng; g0 += 8 * RW) {  // eight groups in flight
+          uint32_t k2[8];
+#pragma unroll
+          for (int z = 0; z < 8; ++z) k2[z] = words(g0 + z * RW);
+#pragma unroll
+          for (int z = 0; z < 8; ++z)
+            if (g0 + z * RW < ng) look(g0 + z * RW, k2[z]);
+        }
+      } else {
+        const int nd = sh.ngrp;
+        for (int k = warp; k < nd; k += RW) look(glist[k], words(glist[k]));
+      }
+      __syncthreads();
+      if (threadIdx.x == 0) sh.ngrp = sh.grp_all = 0;
+      gall = false;
+      marked = 0;
+      unsigned long long best = 0ull;
+      for (int g = threadIdx.x; g < ng; g += RB) {
+        const unsigned b = gbest[g];
+        if (b == 0u) continue;
+        const unsigned id = (unsigned)(g * PICK_GROUP + 63) - ((b - 1u) & 63u);
+        best = max(best, ((unsigned long long)((b - 1u) >> 6) << 32) | (unsigned)~id);
       }
       best = block_best(best, sh);
       X = best ? (int)~(unsigned)best : -1;
@@ -928,6 +980,7 @@ __device__ __noinline__ int2 first_pass(const Mem<IT> *m0, int64_t d, bool ccr, 
       phmin[phases] = X;
       m.F[phases] = comp;
       kh[X] = (uint16_t)KEY_IN;
+      if (GROUPS) glist[sh.ngrp++] = X / PICK_GROUP;
     }
     int head = tail++;
     __syncthreads();
@@ -937,6 +990,7 @@ __device__ __noinline__ int2 first_pass(const Mem<IT> *m0, int64_t d, bool ccr, 
       int32_t *qn = &sh.qn[r];
       const int rn = r == 2 ? 0 : r + 1;
       if (threadIdx.x == 0) sh.qn[rn] = 0;
+      if (GROUPS && (F > RW || ++marked > PICK_ROUNDS)) gall = true;
       if (F >= PULL_MIN && F >= U) {
         // every unadded vertex counts its added neighbours afresh; those it
         // takes are marked only after the round, so that the keys of the
@@ -988,6 +1042,7 @@ __device__ __noinline__ int2 first_pass(const Mem<IT> *m0, int64_t d, bool ccr, 
       } else {
         // the vertices added last raise their neighbours' keys; loads and
         // atomics of four entries a lane overlap
+        bool mark = false;  // the groups of the vertices raised are listed
         auto raise = [&](const int (&j)[4], int) {
           unsigned k[4], old[4];
           bool take[4];
@@ -1006,11 +1061,25 @@ __device__ __noinline__ int2 first_pass(const Mem<IT> *m0, int64_t d, bool ccr, 
             }
           }
           warp_push4(take, j, queue, tail, qn);
+          if (GROUPS && mark) {
+            bool up[4];
+            int g[4];
+#pragma unroll
+            for (int z = 0; z < 4; ++z) {
+              up[z] = k[z] < (unsigned)kcap;
+              g[z] = j[z] / PICK_GROUP;
+            }
+            warp_push4(up, g, glist, 0, &sh.ngrp);
+          }
         };
         if (F <= RW) {
           if (warp < F) {
-            const int v = queue[head + warp];
-            one_row(m.adj, m.off[v], (int)m.len[v], raise);
+            const int v = queue[head + warp], d = (int)m.len[v];
+            if (GROUPS) {
+              mark = !gall && d <= PICK_ROW;
+              if (!mark && lane == 0) sh.grp_all = 1;
+            }
+            one_row(m.adj, m.off[v], d, raise);
           }
         } else {
           const int per = min(32, (F + RW - 1) / RW);

@@ -257,3 +257,32 @@ def test_a_failed_run_ends_between_kept_parts(wcc, monkeypatch):
         assert time.perf_counter() - t0 < full / 4
         monkeypatch.delenv("WCC_WAIT_LIMIT_MS")
         assert np.array_equal(g.run(w.labels, min_size=w.min_size), ref)
+
+
+def test_picks_by_groups_in_items_with_32bit_local_ids(wcc, monkeypatch):
+    """One cluster of 65,601 vertices (not a multiple of the 64 of a group): a
+    sparse random part, whose pass has thousands of picks, rows around the 256
+    entries whose neighbours are listed by group, and a ring lattice, whose
+    closures grow over more small rounds than are listed and which a cut of three
+    edges splits off.  With the keys in
+    shared memory and in the item's global memory."""
+    rng = np.random.default_rng(9)
+    n, nr = 65_601, 60_000
+    m = int(nr * 11.0 / 2)
+    eu, ev = [rng.integers(0, nr, m)], [rng.integers(0, nr, m)]
+    for h, deg in enumerate((255, 256, 257, 258, 3000)):
+        eu.append(np.full(deg, h)); ev.append(rng.choice(np.arange(10, nr), deg, replace=False))
+    i = np.arange(nr, n)
+    for d in range(1, 6):
+        eu.append(i); ev.append(nr + (i - nr + d) % (n - nr))
+    eu.append(rng.integers(0, nr, 3)); ev.append(rng.integers(nr, n, 3))
+    w = _finish(rng, n, np.concatenate(eu), np.concatenate(ev), np.zeros(n, np.int32), 2, "groups")
+    off, adj = oracle.build_csr(w.n, w.src, w.dst)
+    ref, rst = oracle.wcc(w.n, off, adj, w.labels, w.min_size)
+    with wcc.WccGraph.from_edges(w.src, w.dst, w.n) as g:
+        for kb in (None, "16"):
+            if kb:
+                monkeypatch.setenv("WCC_SMEM_KB", kb)
+            out, st = g.run(w.labels, min_size=w.min_size, stats=True)
+            assert np.array_equal(out, ref)
+            assert st["splits"] == rst["splits"] >= 1
