@@ -22,7 +22,9 @@
 //      dropped, and the result written at the bucket's place;
 //      buckets too large for shared memory are taken by a second kernel that
 //      gathers rows in global memory and splits rows that are themselves too
-//      long by the columns' leading bits;
+//      long by the columns' leading bits; the entries of still larger ones (and
+//      of those with too many equal columns) are sorted together, by the radix
+//      sort;
 //   5. a scan of the rows' degrees gives the offsets; without repeats or loops
 //      the columns are in place already, else one more copy packs them.
 // It moves each entry 5 times (read as an edge twice, written and read as 8
@@ -60,6 +62,11 @@ constexpr int SUB_MAX = ROWS_MAX + 2 * BUCKET_CAP / PART_AVG;  // rows and parts
 constexpr int BB = 512;              // threads of a large bucket's CTA
 constexpr int BIG_CAP = 16384;       // entries it sorts in shared memory at once
 constexpr int BIG_CTAS = 304;
+// Entries of a bucket that one CTA takes; the ones of larger buckets are sorted
+// together.  One row of 20,000 / 50,000 / 99,000 neighbours in 500,000 edges: 0.38 /
+// 0.56 / 0.81 ms by a CTA, 0.30 / 0.31 / 0.33 by the sort; but a thousand buckets of
+// 20,000 keep all CTAs busy: 0.81 ms against 1.16.
+constexpr uint32_t HUGE_CAP = 32768;
 constexpr int SMALL_T = 1024;        // a graph one CTA builds alone: its threads,
 constexpr int SMALL_ROWS = 4096;     // rows
 constexpr int SMALL_ENTRIES = 12 * 1024;  // and directed entries
@@ -69,7 +76,7 @@ constexpr size_t SMALL_SMEM = 4 * (size_t)(2 * SMALL_ROWS + 1 + SMALL_ENTRIES);
 
 // What a build reports back in one copy.
 struct Result {
-  unsigned err, big, over;  // DERR_* bits, large buckets, a bucket or part too long
+  unsigned err, big, huge;  // DERR_* bits, large buckets, those left to the radix sort
   uint32_t placed;          // entries in the buckets (the loops' excluded)
   int64_t nnz;
 };
@@ -427,7 +434,7 @@ __device__ __forceinline__ int part_bits(int len) {
 __global__ void __launch_bounds__(SB) k_bucket_sort(Plan p, const uint32_t *__restrict__ in,
                                                    const uint32_t *__restrict__ start,
                                                    uint32_t *out, int64_t *deg, uint32_t *big,
-                                                   Result *res) {
+                                                   uint32_t *huge, Result *res) {
   extern __shared__ __align__(16) unsigned char smem[];
   uint32_t *buf = reinterpret_cast<uint32_t *>(smem);
   __shared__ uint32_t cnt[SUB_MAX], rs[SUB_MAX + 1], us[SUB_MAX + 1];
@@ -442,8 +449,8 @@ __global__ void __launch_bounds__(SB) k_bucket_sort(Plan p, const uint32_t *__re
   if (threadIdx.x == 0 && q == p.nb - 1) res->placed = start[p.nb];
   if (entries > (uint32_t)BUCKET_CAP) {
     if (threadIdx.x == 0) {
-      if (entries > (uint32_t)INT32_MAX)
-        res->over = 1u;
+      if (entries > HUGE_CAP)
+        huge[atomicAdd(&res->huge, 1u)] = q;
       else
         big[atomicAdd(&res->big, 1u)] = q;
     }
@@ -599,12 +606,13 @@ __device__ __forceinline__ int sort_by_parts(const uint32_t *from, int len, uint
 // The listed buckets, by whole CTAs in global memory: rows gathered into alt,
 // then sorted there: short ones by warps, rows of up to BIG_CAP entries in
 // shared memory, longer ones split by the columns' top bits into at most 256
-// parts through out and sorted part by part.  A part above BIG_CAP sets
-// over: the caller builds with the full sort.
+// parts through out and sorted part by part.  A bucket with a part above
+// BIG_CAP is left to the radix sort.
 __global__ void __launch_bounds__(BB) k_bucket_big(Plan p, const uint32_t *in,
                                                   const uint32_t *__restrict__ start, uint32_t *alt,
                                                   uint32_t *out, int64_t *deg,
-                                                  const uint32_t *__restrict__ big, Result *res) {
+                                                  const uint32_t *__restrict__ big,
+                                                  uint32_t *huge, Result *res) {
   extern __shared__ __align__(16) unsigned char smem[];
   uint32_t *buf = reinterpret_cast<uint32_t *>(smem);
   __shared__ uint32_t cnt[ROWS_MAX], rs[ROWS_MAX + 1], us[ROWS_MAX + 1];
@@ -659,7 +667,8 @@ __global__ void __launch_bounds__(BB) k_bucket_big(Plan p, const uint32_t *in,
       if (lane == 0) cnt[r] = (uint32_t)d;
     }
     __syncthreads();
-    for (int r = 0; r < rows; ++r) {
+    bool over = false;
+    for (int r = 0; r < rows && !over; ++r) {
       const uint32_t len = rs[r + 1] - rs[r];
       if (len <= (uint32_t)ROW_WARP) continue;
       uint32_t *row = ab + rs[r];
@@ -674,11 +683,8 @@ __global__ void __launch_bounds__(BB) k_bucket_big(Plan p, const uint32_t *in,
           int g1 = g0 + 1;
           while (g1 < 256 && ps[g1 + 1] - ps[g0] <= (uint32_t)BIG_CAP) ++g1;
           const uint32_t a = ps[g0], l = ps[g1] - a;
-          if (l > (uint32_t)BIG_CAP) {
-            if (threadIdx.x == 0) res->over = 1u;
-            g0 = g1;
-            continue;
-          }
+          over = l > (uint32_t)BIG_CAP;
+          if (over) break;
           d += (uint32_t)sort_by_parts<BB>(ob + rs[r] + a, (int)l, (uint32_t)g0 << vshift,
                                            (uint32_t)(g1 - g0) << vshift, buf, row + d, sp);
           g0 = g1;
@@ -686,6 +692,10 @@ __global__ void __launch_bounds__(BB) k_bucket_big(Plan p, const uint32_t *in,
       }
       if (threadIdx.x == 0) cnt[r] = d;
       __syncthreads();
+    }
+    if (over) {
+      if (threadIdx.x == 0) huge[atomicAdd(&res->huge, 1u)] = q;
+      continue;
     }
     if (threadIdx.x < ROWS_MAX && threadIdx.x >= rows) cnt[threadIdx.x] = 0;
     __syncthreads();
@@ -806,15 +816,130 @@ __global__ void __launch_bounds__(SMALL_T) k_csr_small(const int32_t *__restrict
   }
 }
 
+// ---- the buckets left to the radix sort ------------------------------------------
+// Bucket k of the list huge[0..count): its entries are hstart[k] .. hstart[k + 1]
+// of all the listed ones'.  One block.
+__global__ void __launch_bounds__(1024) k_huge_starts(const uint32_t *__restrict__ start,
+                                                     const uint32_t *__restrict__ huge,
+                                                     uint32_t count, uint32_t *hstart) {
+  __shared__ uint32_t sm[1024 / 32 + 1];
+  uint32_t carry = 0;
+  for (uint32_t k0 = 0; k0 < count; k0 += 1024) {
+    const uint32_t k = k0 + threadIdx.x;
+    uint32_t tot;
+    const uint32_t ex = block_exclusive_scan<1024>(
+        k < count ? start[huge[k] + 1] - start[huge[k]] : 0u, &tot, sm);
+    if (k < count) hstart[k] = carry + ex;
+    carry += tot;
+  }
+  if (threadIdx.x == 0) hstart[count] = carry;
+}
+
+// keys[i] = (k, entry) of the listed buckets' entry i, in bucket k.
+__global__ void k_huge_keys(Plan p, const uint32_t *__restrict__ in,
+                            const uint32_t *__restrict__ start, const uint32_t *__restrict__ huge,
+                            uint32_t count, const uint32_t *__restrict__ hstart, int64_t total,
+                            uint64_t *keys) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= total) return;
+  uint32_t lo = 0, hi = count - 1;  // the last k with hstart[k] <= i
+  while (lo < hi) {
+    const uint32_t mid = (lo + hi + 1) >> 1;
+    if (hstart[mid] <= (uint32_t)i) lo = mid; else hi = mid - 1;
+  }
+  keys[i] = ((uint64_t)lo << (p.b + p.s)) | in[start[huge[lo]] + ((uint32_t)i - hstart[lo])];
+}
+
+__global__ void k_huge_first(const uint64_t *__restrict__ keys, int64_t total, uint32_t *keep) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < total) keep[i] = i == 0 || keys[i - 1] != keys[i] ? 1u : 0u;
+}
+
+// deg[r] = the columns of row r by the offsets; 0 in the listed buckets (block
+// = rows of one bucket).
+__global__ void k_huge_degrees(const int64_t *__restrict__ off, int64_t n, int64_t *deg) {
+  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (r < n) deg[r] = off[r + 1] - off[r];
+}
+__global__ void __launch_bounds__(ROWS_MAX) k_huge_clear(Plan p, const uint32_t *__restrict__ huge,
+                                                        int64_t *deg) {
+  const int64_t r = ((int64_t)huge[blockIdx.x] << p.s) + threadIdx.x;
+  if (threadIdx.x < (1 << p.s) && r < p.n) deg[r] = 0;
+}
+
+// The first copies in order to their bucket's place in out, and their rows'
+// degrees (sorted keys: one atomic per row and warp).
+__global__ void k_huge_write(Plan p, const uint64_t *__restrict__ keys,
+                             const uint32_t *__restrict__ keep, const uint32_t *__restrict__ pos,
+                             int64_t total, const uint32_t *__restrict__ start,
+                             const uint32_t *__restrict__ huge, const uint32_t *__restrict__ hstart,
+                             uint32_t *out, int64_t *deg) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool kept = i < total && keep[i];
+  int64_t row = -1;
+  if (kept) {
+    const uint32_t k = (uint32_t)(keys[i] >> (p.b + p.s)), q = huge[k];
+    const uint64_t e = keys[i] & ((1ull << (p.b + p.s)) - 1);
+    row = ((int64_t)q << p.s) + (int64_t)(e >> p.b);
+    out[start[q] + (pos[i] - pos[hstart[k]])] = (uint32_t)(e & ((1ull << p.b) - 1));
+  }
+  const unsigned peers = __match_any_sync(FULL, (unsigned long long)row);
+  if (kept && (peers & lanemask_lt()) == 0u)
+    atomicAdd((unsigned long long *)&deg[row], (unsigned long long)__popc(peers));
+}
+
 // With repeats or loops dropped: every bucket's columns to their final place.
+// Those above HUGE_CAP (list: huge) by PACK_CTAS CTAs each, the others by one.
+constexpr unsigned PACK_CTAS = 64;
 __global__ void __launch_bounds__(SB) k_bucket_pack(Plan p, const uint32_t *__restrict__ in,
                                                    const uint32_t *__restrict__ start,
+                                                   const uint32_t *__restrict__ huge,
                                                    const int64_t *__restrict__ off, int32_t *adj) {
-  const uint32_t q = blockIdx.x;
+  const uint32_t q = huge ? huge[blockIdx.x] : blockIdx.x;
+  const uint32_t from = start[q];
+  if ((start[q + 1] - from > HUGE_CAP) != (huge != nullptr)) return;
   const int64_t r0 = (int64_t)q << p.s, r1 = min(r0 + ((int64_t)1 << p.s), p.n);
-  const int64_t to = off[r0];
-  const uint32_t len = (uint32_t)(off[r1] - to), from = start[q];
-  for (uint32_t i = threadIdx.x; i < len; i += SB) adj[to + i] = (int32_t)in[from + i];
+  const int64_t to = off[r0], len = off[r1] - to;
+  for (int64_t i = (int64_t)blockIdx.y * SB + threadIdx.x; i < len; i += gridDim.y * SB)
+    adj[to + i] = (int32_t)in[from + i];
+}
+
+// Sorts the entries of the huge listed buckets all at once, writes their
+// columns and makes the offsets anew.  keys: 64-bit memory that may be
+// overwritten (grown when it is too small); in: their entries, overwritten too.
+// A row of 1,900,000 neighbours in 20M edges: 1.46 ms in all (one CTA taking the
+// bucket 12.9, one CTA packing it 2.38; the full sort of all entries 3.5).
+Result sort_huge(const Plan &p, uint32_t *in, const uint32_t *start, const uint32_t *huge,
+                 uint32_t count, uint32_t *out, int64_t *off, DevBuf &keys, DevBuf &temp,
+                 Result *res, cudaStream_t s) {
+  DevBuf bstart, bkeys2, bpos, bdeg;
+  uint32_t *hstart = static_cast<uint32_t *>(bstart.ensure(4 * ((size_t)count + 1)));
+  k_huge_starts<<<1, 1024, 0, s>>>(start, huge, count, hstart); note_launch();
+  WCC_CUDA(cudaGetLastError());
+  const int64_t total = read_back(hstart + count, s);
+  uint64_t *k1 = static_cast<uint64_t *>(keys.ensure(8 * (size_t)total));
+  uint64_t *k2 = static_cast<uint64_t *>(bkeys2.ensure(8 * (size_t)total));
+  uint32_t *pos = static_cast<uint32_t *>(bpos.ensure(4 * ((size_t)total + 1)));
+  int64_t *deg = static_cast<int64_t *>(bdeg.ensure(8 * (size_t)(p.n + 1)));
+  void *t = temp.ensure(std::max({radix_temp_bytes(total), scan_temp_bytes(total + 1),
+                                  scan_temp_bytes(p.n + 1)}) + 64);
+  const unsigned g = grid_for(total);
+  k_huge_keys<<<g, SB, 0, s>>>(p, in, start, huge, count, hstart, total, k1); note_launch();
+  WCC_CUDA(cudaGetLastError());
+  const int bits = p.b + p.s + (int)bitlen_u64(count - 1);
+  const uint64_t *sorted = radix_sort_keys_u64(k1, k2, total, bits, t, &res->err, s) ? k2 : k1;
+  if (read_back(&res->err, s)) fail(WCC_ERR_TIMEOUT, "CSR build: a bounded wait of the sort ran out");
+  uint32_t *keep = in;
+  k_huge_first<<<g, SB, 0, s>>>(sorted, total, keep); note_launch();
+  exclusive_scan_u32(keep, pos, total, pos + total, t, s);
+  k_huge_degrees<<<grid_for(p.n), SB, 0, s>>>(off, p.n, deg); note_launch();
+  k_huge_clear<<<count, ROWS_MAX, 0, s>>>(p, huge, deg); note_launch();
+  k_huge_write<<<g, SB, 0, s>>>(p, sorted, keep, pos, total, start, huge, hstart, out, deg);
+  note_launch();
+  WCC_CUDA(cudaMemsetAsync(deg + p.n, 0, 8, s));
+  exclusive_scan_i64(deg, off, p.n + 1, &res->nnz, t, s);
+  WCC_CUDA(cudaGetLastError());
+  return read_back(res, s);  // (the buffers above are given back only after it)
 }
 
 }  // namespace
@@ -844,7 +969,8 @@ bool csr_by_buckets(const int32_t *src, const int32_t *dst, int64_t m, int64_t n
   while (p.s < 8 && p.b + p.s + 1 <= 32 && (n2 << (p.s + 1)) <= (int64_t)BUCKET_AVG * std::max<int64_t>(n, 1))
     ++p.s;
   const int64_t nb = n > 0 ? ((n - 1) >> p.s) + 1 : 0;
-  if (nb + 1 > (int64_t)BIN_MAX * BIN_MAX) return false;
+  // too many buckets, or (copies of few edges) all of them huge
+  if (nb + 1 > (int64_t)BIN_MAX * BIN_MAX || n2 > (int64_t)HUGE_CAP * nb) return false;
   p.nb = (unsigned)nb;
   if (nb + 1 > BIN_MAX) {
     const int bits = (int)bitlen_u64((uint64_t)nb);
@@ -868,7 +994,8 @@ bool csr_by_buckets(const int32_t *src, const int32_t *dst, int64_t m, int64_t n
   uint32_t *cur1 = start1 + BIN_MAX + 1, *tile0 = cur1 + BIN_MAX + 1;
   uint16_t *owner = reinterpret_cast<uint16_t *>(tile0 + BIN_MAX + 1);
   void *temp = w[4].ensure(std::max(scan_temp_bytes((int64_t)nq + 1), scan_temp_bytes(n + 1)) + 64);
-  uint32_t *big = static_cast<uint32_t *>(w[5].ensure(4 * (size_t)std::max<int64_t>(nb, 1)));
+  uint32_t *big = static_cast<uint32_t *>(w[5].ensure(8 * (size_t)std::max<int64_t>(nb, 1)));
+  uint32_t *huge = big + nb;
   // the 64-bit entries of the first partition; later the large buckets' rows
   uint64_t *k64 = static_cast<uint64_t *>(w[6].ensure((two ? 8 : 4) * (size_t)n2));
   uint32_t *k32 = static_cast<uint32_t *>(w[7].ensure(4 * (size_t)n2));
@@ -905,23 +1032,27 @@ bool csr_by_buckets(const int32_t *src, const int32_t *dst, int64_t m, int64_t n
   }
   WCC_CUDA(cudaGetLastError());
   if (nb > 0) {
-    k_bucket_sort<<<(unsigned)nb, SB, smb, s>>>(p, k32, start, adj, off, big, res);
+    k_bucket_sort<<<(unsigned)nb, SB, smb, s>>>(p, k32, start, adj, off, big, huge, res);
     note_launch();
     k_bucket_big<<<(unsigned)std::min<int64_t>(nb, BIG_CTAS), BB, smg, s>>>(
-        p, k32, start, reinterpret_cast<uint32_t *>(k64), adj, off, big, res);
+        p, k32, start, reinterpret_cast<uint32_t *>(k64), adj, off, big, huge, res);
     note_launch();
   }
   WCC_CUDA(cudaMemsetAsync(off + n, 0, 8, s));
   exclusive_scan_i64(off, off, n + 1, &res->nnz, temp, s);
   WCC_CUDA(cudaGetLastError());
-  const Result r = read_back(res, s);
+  Result r = read_back(res, s);
   if (r.err & DERR_INVALID) fail(WCC_ERR_INVALID, "edge endpoint outside [0, n)");
-  if (r.over) return false;
+  if (r.huge > 0) r = sort_huge(p, k32, start, huge, r.huge, adj, off, w[6], w[4], res, s);
   const int64_t nnz = r.nnz;
   if (nnz != (int64_t)r.placed) {
     // repeats were dropped: the buckets' columns close up, into k32's memory
-    k_bucket_pack<<<(unsigned)nb, SB, 0, s>>>(p, adj, start, off, reinterpret_cast<int32_t *>(k32));
-    note_launch();
+    int32_t *to = reinterpret_cast<int32_t *>(k32);
+    k_bucket_pack<<<(unsigned)nb, SB, 0, s>>>(p, adj, start, nullptr, off, to); note_launch();
+    if (r.huge > 0) {
+      k_bucket_pack<<<dim3(r.huge, PACK_CTAS), SB, 0, s>>>(p, adj, start, huge, off, to);
+      note_launch();
+    }
     WCC_CUDA(cudaGetLastError());
     std::swap(adj_buf.p, w[7].p);
     std::swap(adj_buf.bytes, w[7].bytes);

@@ -65,11 +65,12 @@ struct Workspace {
 // ---- csr.cu ----------------------------------------------------------------
 // CSR of an edge list by buckets of rows (partition, sort every bucket on
 // chip).  Fills off[0..n] and adj_buf and returns true; returns false, leaving
-// both with unspecified contents, when the graph has too many buckets (above
-// about 2^28 rows, fewer with more than 2^24) or a part of a row that is too
-// long to sort on chip (the caller then sorts all entries).  An endpoint
-// outside [0, n) fails with WCC_ERR_INVALID.  `w`: its temporaries, grown on
-// demand.
+// both with unspecified contents, when the caller has to sort all entries: the
+// graph has too many buckets (more than 2^20 - 1: from just under 2^26 rows on,
+// where a row and a column no longer fit 32 bits with fewer, or with more than
+// about 2.7 billion entries), or so few rows for its entries that all buckets are
+// large.  An endpoint outside [0, n) fails with WCC_ERR_INVALID.  `w`: its
+// temporaries, grown on demand.
 constexpr int CSR_BUCKET_BUFS = 8;
 bool csr_by_buckets(const int32_t *src, const int32_t *dst, int64_t m, int64_t n, int64_t *off,
                     DevBuf &adj_buf, int64_t *nnz_out, DevBuf (&w)[CSR_BUCKET_BUFS],

@@ -86,6 +86,41 @@ def test_builder_refuses_endpoints_out_of_range(n, m, bad):
         wcc.WccGraph.from_edges(u.astype(np.int32), v.astype(np.int32), n)
 
 
+HUGE = 32_768  # entries of a bucket that one CTA takes; more are sorted together
+HUGE_CASES = {
+    # rows (a bucket of their own entries and few more) around the limit
+    "rows": (300_000, *_hubs(300_000, 400_000, [HUGE - 300, HUGE - 1, HUGE, HUGE + 1, 70_000], 31)),
+    # one digit, two digits; one huge bucket, many, hubs in the last rows
+    "one_digit": (100_000, *_hubs(100_000, 300_000, [99_000], 32)),
+    "many": (400_000, *_hubs(400_000, 500_000, [60_000 + 1000 * k for k in range(12)], 33)),
+    "last_rows": (300_000, *(299_999 - x for x in _hubs(300_000, 200_000, [200_000, 40_000], 34))),
+    "star": (250_000, np.zeros(249_999, np.int64), np.arange(1, 250_000)),
+    # equal columns past what a CTA sorts: below the limit, and above with loops and repeats
+    "copies_below": (30_000, *(np.concatenate([np.full(17_000, a), b]) for a, b in
+                               zip((7, 9), _random(30_000, 30_000, 35)))),
+    "copies_above": (30_000, *(np.concatenate([np.full(90_000, a), np.full(300, 5), b]) for a, b in
+                               zip((7, 9), _random(30_000, 30_000, 36)))),
+    # nearly every bucket huge; all of them (the full sort of all entries)
+    "dense": (70, *_random(70, 1_146_000, 37)),
+    "dense_over": (70, *_random(70, 1_200_000, 38)),
+}
+
+
+@pytest.mark.parametrize("name", list(HUGE_CASES))
+def test_huge_buckets_equal_oracle(name):
+    import paper_2509_02590_gb300 as wcc
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    n, u, v = HUGE_CASES[name]
+    for seed in (None, 1):  # as they are, and shuffled
+        p = np.arange(len(u)) if seed is None else np.random.default_rng(seed).permutation(len(u))
+        src, dst = u[p].astype(np.int32), v[p].astype(np.int32)
+        off, adj = oracle.build_csr(n, src, dst)
+        with wcc.WccGraph.from_edges(torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda(), n) as g:
+            goff, gadj = g.csr()
+        assert np.array_equal(goff, off) and np.array_equal(gadj, adj)
+
+
 def _copies_of_one_edge(extra):
     """2^30 + extra edges on 900,000 vertices, all but 5,000 of them 0-1: more
     than 2^31 entries in the first bucket, which holds rows 0 and 1.  Run in a
