@@ -2865,6 +2865,7 @@ __global__ void __launch_bounds__(RB, 1) k_refine(RefineParams P) {
         sh.bdone = 0;
         sh.ncta = 0;
       }
+      __syncwarp();  // lane 0 has read the last batch's statistics
       if (lane < 7) sh.tst[lane] = 0ull;
     }
     __syncthreads();

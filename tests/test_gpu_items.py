@@ -286,3 +286,27 @@ def test_picks_by_groups_in_items_with_32bit_local_ids(wcc, monkeypatch):
             out, st = g.run(w.labels, min_size=w.min_size, stats=True)
             assert np.array_equal(out, ref)
             assert st["splits"] == rst["splits"] >= 1
+
+
+def test_statistics_of_batches_of_small_items(wcc):
+    """The counters that the warps of a batch of small items add up are read by
+    one lane before the others clear them for the next batch: totals over 6,000
+    clusters of 5-40 vertices, taken in many batches, in every one of 30 runs."""
+    rng = np.random.default_rng(12)
+    eu, ev, lab, n = [], [], [], 0
+    for c in range(6000):
+        size = int(rng.integers(5, 41))
+        iu, ju = np.triu_indices(size, 1)
+        keep = rng.random(len(iu)) < rng.uniform(0.1, 0.6)
+        eu.append(n + iu[keep]); ev.append(n + ju[keep]); lab.append(np.full(size, c))
+        n += size
+    w = _finish(rng, n, np.concatenate(eu), np.concatenate(ev), np.concatenate(lab), 2, "small items")
+    off, adj = oracle.build_csr(w.n, w.src, w.dst)
+    ref, rst = oracle.wcc(w.n, off, adj, w.labels, w.min_size)
+    want = {k: rst[k] for k in ("in_clusters", "out_clusters", "splits", "peeled")}
+    lab_dev = torch.from_numpy(w.labels).cuda()
+    with wcc.WccGraph.from_edges(w.src, w.dst, w.n) as g:
+        for _ in range(30):
+            out, st = g.run(lab_dev, min_size=w.min_size, stats=True)
+            assert {k: st[k] for k in want} == want
+    assert np.array_equal(out.cpu().numpy(), ref)
