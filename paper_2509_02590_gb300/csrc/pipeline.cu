@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(GT) k_group_small(const int32_t *__restrict__ 
     if (i < n) {
       const int32_t c = lab[i];
       if (c < -1) bad = 1u;
-      key = ((unsigned long long)(unsigned)(c + 1) << 32) | (unsigned)i;
+      key = ((unsigned long long)((unsigned)c + 1u) << 32) | (unsigned)i;
     }
     a[i] = key;
   }
