@@ -385,6 +385,19 @@ enum RunBuf { R_IN, R_OUT, R_POOL, R_SLOT, R_LMIN, R_RING, R_CTR, R_SLAB, R_INH,
               R_CM_PARTS, R_CM_PARTOF, R_CM_SCRATCH, R_CM_ITEMS, R_CM_MISC, R_COUNT };
 static_assert(R_COUNT <= 16, "Graph::rb holds 16 buffers");
 
+// Whether kernels on dev can write int32 values at p: aligned memory of that
+// device, or managed.  Whatever else a copy accepts (an address that is not
+// aligned, another device's or pinned host memory) is written by a copy.
+bool kernels_can_write(const void *p, int dev) {
+  cudaPointerAttributes a{};
+  if (reinterpret_cast<uintptr_t>(p) % alignof(int32_t) != 0) return false;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == dev);
+}
+
 // What a run reads back at its end, in one copy.
 struct RunEnd {
   RunCounters ctr;
@@ -541,14 +554,16 @@ void run_impl(Graph *g, const int32_t *lab_in, const wcc_threshold_rule *rule, i
   tm.mark(2, s);
   // ---- a9: ids = rank of each accepted cluster's smallest vertex, numbered
   // right behind the kernel; a run that failed writes none of them
-  int32_t *d_out = on_device ? lab_out : static_cast<int32_t *>(rb[R_OUT].ensure(4 * n));
+  const bool direct = on_device && kernels_can_write(lab_out, dev);
+  int32_t *d_out = direct ? lab_out : static_cast<int32_t *>(rb[R_OUT].ensure(4 * n));
   number_clusters(lmin, n, d_out, g->ws, s, &ctr->error);
   tm.mark(3, s);
   const RunEnd he = read_back(end, s);
   const ReqCtx &hr = he.req;
   check_derr(he.ctr.error, "refinement");
-  if (!on_device) {
-    WCC_CUDA(cudaMemcpyAsync(lab_out, d_out, 4 * n, cudaMemcpyDeviceToHost, s));
+  if (!direct) {
+    WCC_CUDA(cudaMemcpyAsync(lab_out, d_out, 4 * n,
+                             on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
     WCC_CUDA(cudaStreamSynchronize(s));
   }
 

@@ -59,3 +59,29 @@ def test_labels_below_minus_one_are_refused(n):
     with wcc.WccGraph.from_edges(np.array([0], np.int32), np.array([1], np.int32), n) as g:
         with pytest.raises(wcc.WccError):
             g.run(lab)
+
+
+@pytest.mark.parametrize("n", [1000, 9000])
+def test_device_output_that_only_a_copy_can_write(n):
+    """clustering_out on the device path is written by the numbering kernel when
+    it can; an address that is not aligned, or pinned host memory, takes a copy."""
+    import paper_2509_02590_gb300 as wcc
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    w = synth.lfr_like(n, seed=3)
+    lab = torch.from_numpy(w.labels).cuda()
+    stream = torch.cuda.current_stream().cuda_stream
+    with wcc.WccGraph.from_edges(w.src, w.dst, w.n) as g:
+        ref = g.run(lab).cpu().numpy()
+        for shift in (1, 2, 3):
+            raw = torch.full((4 * n + 8,), 7, dtype=torch.uint8, device="cuda")
+            torch.cuda.synchronize()
+            wcc.wcc_run(g.handle, lab.data_ptr(), wcc.rule_struct(), 2, wcc.WCC_MODE_BATCHED,
+                        raw.data_ptr() + shift, 1, stream, None)
+            got = raw.cpu().numpy()
+            assert np.array_equal(got[shift:shift + 4 * n].copy().view(np.int32), ref)
+            assert (got[:shift] == 7).all() and (got[shift + 4 * n:] == 7).all()
+        pinned = torch.empty(n, dtype=torch.int32).pin_memory()
+        wcc.wcc_run(g.handle, lab.data_ptr(), wcc.rule_struct(), 2, wcc.WCC_MODE_BATCHED,
+                    pinned.data_ptr(), 1, stream, None)
+        assert np.array_equal(pinned.numpy(), ref)
