@@ -2984,7 +2984,8 @@ __global__ void __launch_bounds__(RB, 1) k_refine(RefineParams P) {
       }
       if (threadIdx.x == 0) {
         finish_items(P, it.req, 1);
-        sh.go = vctr->error == 0;
+        // (only a chain needs it: the next claim looks too)
+        if (sh.has_own) sh.go = vctr->error == 0;
       }
       __syncthreads();
       if (!sh.go) break;  // the run has failed: a chain of kept parts ends too
