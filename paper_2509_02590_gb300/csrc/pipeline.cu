@@ -29,9 +29,14 @@ struct SeedInfo {
 };
 
 // Graphs of at most GROUP_SMALL vertices are grouped, seeded and numbered by
-// one CTA each (see k_group_small).
-constexpr int GROUP_SMALL = 8192;
+// one CTA each (see k_group_small), whose sorting network grows with the vertices
+// while the launches it saves do not.  Whole runs, one CTA / the general path, two
+// kinds of graph: 1,000 vertices 0.132, 0.144 / 0.174, 0.188 ms; 2,000 0.147, 0.208 /
+// 0.182, 0.212; 3,000 0.167, 0.307 / 0.184, 0.269; 4,096 0.187, 0.347 / 0.191, 0.284;
+// 8,192 0.246, 0.488 / 0.212, 0.362.
+constexpr int GROUP_SMALL = 2048;
 constexpr int GT = 1024;  // its threads
+static_assert(8 * GROUP_SMALL <= 32 * 1024, "its keys fit the shared memory of any launch");
 
 // keys[v] = label + 1 (0 for unclustered), vals[v] = v; largest key; labels
 // below -1 are malformed.
@@ -551,9 +556,6 @@ GroupInfo group_by_label(const int64_t *off, int64_t n, const int32_t *labels, i
     SeedInfo *info = buf<SeedInfo>(ws, B_INFO, 1);
     size_t P = 2;
     while ((int64_t)P < n) P <<= 1;
-    if (8 * P > 32 * 1024)
-      WCC_CUDA(cudaFuncSetAttribute(k_group_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    8 * GROUP_SMALL));
     k_group_small<<<1, GT, 8 * P, s>>>(labels, (int)n, off, min_size, vals, cl, cstart, keep, qidx,
                                        info);
     note_launch();

@@ -1,5 +1,5 @@
 """Grouping, seeding and numbering at the sizes where they change form: one CTA
-up to 8,192 vertices, tiles of 2,048 sorted positions above, the queue order by
+up to 2,048 vertices, tiles of 2,048 sorted positions above, the queue order by
 one block up to 4,096 clusters.  The refinement's result must be the oracle's."""
 import numpy as np
 import pytest
@@ -85,3 +85,9 @@ def test_device_output_that_only_a_copy_can_write(n):
         wcc.wcc_run(g.handle, lab.data_ptr(), wcc.rule_struct(), 2, wcc.WCC_MODE_BATCHED,
                     pinned.data_ptr(), 1, stream, None)
         assert np.array_equal(pinned.numpy(), ref)
+
+
+@pytest.mark.parametrize("n", [2047, 2048, 2049, 4095, 4096, 4097])
+@pytest.mark.parametrize("kind", ["none", "one", "distinct", "pairs", "mixed"])
+def test_sizes_around_the_one_cta_limit(n, kind):
+    test_sizes(n, kind)
