@@ -287,12 +287,13 @@ __global__ void k_unique_flags(const uint64_t *__restrict__ keys, int64_t n2, ui
 }
 
 // The kept entries in order, and the degree of every row.  Keys are sorted,
-// so a warp's entries mostly share a row: one atomic per row and warp.
+// so a warp's entries mostly share a row: one atomic per row and warp.  (After a
+// sort whose wait ran out they are any values; the host fails the call later.)
 __global__ void k_compact_edges(const uint64_t *__restrict__ keys, const uint32_t *__restrict__ keep,
-                                const uint32_t *__restrict__ pos, int64_t n2, int b,
+                                const uint32_t *__restrict__ pos, int64_t n2, int64_t n, int b,
                                 int32_t *cols, int64_t *deg) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool kept = i < n2 && keep[i];
+  const bool kept = i < n2 && keep[i] && (keys[i] >> b) < (uint64_t)n;
   const uint64_t k = kept ? keys[i] : 0ull;
   const unsigned long long u = kept ? (unsigned long long)(k >> b) : ~0ull;
   if (kept) cols[pos[i]] = (int32_t)(k & ((1ull << b) - 1));
@@ -673,7 +674,7 @@ Graph *build_from_edges(const int32_t *src, const int32_t *dst, int64_t m, int64
     k_unique_flags<<<blocks_for(n2), TB, 0, s>>>(sorted, n2, keep, ~0ull); note_launch();
     exclusive_scan_u32(keep, pos, n2, pos + n2, temp, s);
     int32_t *d_adj = static_cast<int32_t *>(g->adj.ensure(4 * n2));
-    k_compact_edges<<<blocks_for(n2), TB, 0, s>>>(sorted, keep, pos, n2, b, d_adj, d_off);
+    k_compact_edges<<<blocks_for(n2), TB, 0, s>>>(sorted, keep, pos, n2, n, b, d_adj, d_off);
     note_launch();
     exclusive_scan_i64(d_off, d_off, n + 1, nullptr, temp, s);
     WCC_CUDA(cudaGetLastError());
@@ -764,7 +765,7 @@ void build_csr_no_alloc(const int32_t *src, const int32_t *dst, int64_t m, int64
     uint64_t *sorted = radix_sort_keys_u64(k1, k2, n2, 2 * b, temp, err, s) ? k2 : k1;
     k_unique_flags<<<blocks_for(n2), TB, 0, s>>>(sorted, n2, keep, ~0ull); note_launch();
     exclusive_scan_u32(keep, pos, n2, pos + n2, temp, s);
-    k_compact_edges<<<blocks_for(n2), TB, 0, s>>>(sorted, keep, pos, n2, b, cols, row_off);
+    k_compact_edges<<<blocks_for(n2), TB, 0, s>>>(sorted, keep, pos, n2, n, b, cols, row_off);
     note_launch();
     exclusive_scan_i64(row_off, row_off, n + 1, nullptr, temp, s);
     WCC_CUDA(cudaGetLastError());

@@ -114,7 +114,8 @@ __global__ void __launch_bounds__(TB) k_clusters(const uint32_t *__restrict__ sk
 #pragma unroll
   for (int z = 0; z < CI; ++z) {
     const uint32_t v = base + z < n && k[z] ? sv[base + z] : 0u;
-    deg[z] = base + z < n && k[z] ? off[v + 1] - off[v] : 0;
+    // (v is any value after a sort whose wait ran out; the host fails the call later)
+    deg[z] = base + z < n && k[z] && (int64_t)v < n ? off[v + 1] - off[v] : 0;
   }
   unsigned first = 0u;
 #pragma unroll
@@ -138,7 +139,7 @@ __global__ void __launch_bounds__(TB) k_clusters(const uint32_t *__restrict__ sk
     const int64_t i = base + z;
     if (i >= n) break;
     if ((first >> z) & 1u) {
-      if (sum) atomicAdd(&dsum[c], (unsigned long long)sum);
+      if (sum && c >= 0) atomicAdd(&dsum[c], (unsigned long long)sum);
       sum = 0;
       ++c;
       cstart[c] = i;
@@ -154,7 +155,7 @@ __global__ void __launch_bounds__(TB) k_clusters(const uint32_t *__restrict__ sk
     sum = warp_sum(sum);
     if ((threadIdx.x & 31) != 0) sum = 0;
   }
-  if (sum) atomicAdd(&dsum[c], (unsigned long long)sum);
+  if (sum && c >= 0) atomicAdd(&dsum[c], (unsigned long long)sum);
   if (threadIdx.x == 0 && tile == (n - 1) / CTILE) {
     const int64_t K = (int64_t)before_sh + tot;
     cstart[K] = n;
@@ -343,9 +344,10 @@ __global__ void __launch_bounds__(1024) k_order_small(const int64_t *__restrict_
   for (int i = threadIdx.x; i < nkept; i += blockDim.x) qidx[(uint32_t)a[i]] = (uint32_t)i;
 }
 
-__global__ void k_invert(const uint32_t *__restrict__ order, int64_t nkept, uint32_t *qidx) {
+__global__ void k_invert(const uint32_t *__restrict__ order, int64_t nkept, int64_t K,
+                         uint32_t *qidx) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < nkept) qidx[order[i]] = (uint32_t)i;
+  if (i < nkept && order[i] < K) qidx[order[i]] = (uint32_t)i;  // (any value after a failed sort)
 }
 
 // Reserves queue indices [base, base + nkept) for the items of one request
@@ -611,7 +613,7 @@ GroupInfo group_by_label(const int64_t *off, int64_t n, const int32_t *labels, i
     if (radix_sort_pairs_u32(ok1, ov1, ok2, ov2, K, (int)bitlen_u64(gi.max_n + 1), temp,
                              &info->err, s))
       ov = ov2;
-    k_invert<<<grid_for(gi.kept), TB, 0, s>>>(ov, gi.kept, qidx); note_launch();
+    k_invert<<<grid_for(gi.kept), TB, 0, s>>>(ov, gi.kept, K, qidx); note_launch();
     WCC_CUDA(cudaGetLastError());
     const unsigned e = read_back(&info->err, s);
     if (e) check_device_error(e, "grouping");
