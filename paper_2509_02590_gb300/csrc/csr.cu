@@ -50,13 +50,21 @@ constexpr int PT = 512;              // threads of a partition CTA
 constexpr int PK = 16;               // entries a thread
 constexpr int TILE = PT * PK;        // entries a tile
 constexpr int BIN_MAX = 1024;        // buckets told apart by one digit
-constexpr int BUCKET_AVG = 5120;     // entries a bucket is meant to hold
+// Entries a bucket is meant to hold: 2,560 builds 11.7M raw edges on 1M vertices in
+// 0.79 ms instead of 0.92 (fewer of them outgrow a CTA's shared memory) but 53M on
+// 3M vertices in 2.94 instead of 2.74 (twice as many); with 8,192 both take as long
+// as with 5,120.
+constexpr int BUCKET_AVG = 5120;
 constexpr int BUCKET_CAP = 12288;    // entries a CTA sorts in shared memory
 constexpr int SB = 256;              // threads of a bucket's CTA
-constexpr int ROWS_MAX = 256;        // rows of a bucket
+constexpr int ROWS_MAX = 256;        // rows of a bucket (one a thread of its CTA)
 constexpr int ROW_WARP = 512;        // rows up to this long: one warp, in registers
 constexpr int ROW_PART = 256;        // longer rows are split into parts by their columns' top bits
-constexpr int PART_AVG = 192;        // entries a part is meant to hold
+// Entries a part is meant to hold.  A warp's sorting network costs what its size
+// rounded up to a power of two does: at 96 a part mostly takes the one of 128, at 192
+// that of 256.  96 / 192 / 384: 53M edges on 3M vertices 2.66 / 2.74 / 3.56 ms, 11.7M
+// raw on 1M 0.88 / 0.92 / 1.02.
+constexpr int PART_AVG = 96;
 constexpr int PARTS_MAX = 256;       // parts of one row
 constexpr int SUB_MAX = ROWS_MAX + 2 * BUCKET_CAP / PART_AVG;  // rows and parts of a bucket
 constexpr int BB = 512;              // threads of a large bucket's CTA
