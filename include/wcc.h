@@ -272,7 +272,7 @@ int wcc_build_csr_no_alloc(const int32_t *src, const int32_t *dst, int64_t m, in
 
 /* ---- tuning ------------------------------------------------------------
  * The refinement kernel schedules work items by size: items of at most
- * tiny_max vertices run one per warp (up to 8 per CTA) unless their members'
+ * tiny_max vertices run one per warp (up to 16 per CTA) unless their members'
  * degree sum exceeds tiny_max_deg; larger items run on a whole CTA in shared
  * memory (smem_kb per CTA) or, when they do not fit, in a global slab; after
  * the first contraction pass, at most dense_max super-vertices finish on a

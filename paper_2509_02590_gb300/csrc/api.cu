@@ -173,7 +173,7 @@ int dense_max_config() {
 }
 
 // Items of at most this many vertices (WCC_TINY_N, at most 64; 0 keeps every
-// item on a whole CTA) are refined one per warp, up to 8 at once per CTA.
+// item on a whole CTA) are refined one per warp, all warps of a CTA at once.
 int tiny_max_config() {
   const long long v = env_or("WCC_TINY_N", current_tuning().tiny_max);
   return (int)(v < 0 ? 0 : v > 64 ? 64 : v);

@@ -877,9 +877,10 @@ __device__ __forceinline__ void warp_push4(const bool (&take)[4], const int (&v)
 // component, -1 if dead; past MAX_COMP the pass gives up (-2).  With kcap = 1
 // the phases are the components; a pass run for them alone (ccr: rep is B)
 // gives up on long thin items too.  Uses C, D, F, G, H and the keys.  Keys are
-// 16 bits (an increment past kcap is possible while several threads hit one
-// vertex, at most one per thread, so a half-word never overflows into the
-// other).
+// 16 bits: several threads may raise one vertex past kcap, each by up to the four
+// entries it has in flight, which stays below KEY_IN and so out of the other
+// half-word.
+static_assert(KEY_MAX + 4 * RB < (int)KEY_IN, "a key raised past the cap keeps to its half-word");
 template <typename IT, bool SM>
 __device__ __noinline__ int2 first_pass(const Mem<IT> *m0, int64_t d, bool ccr, int n, int nalive,
                                         int kcap, unsigned *err, Sh *shp) {
