@@ -121,6 +121,23 @@ def test_huge_buckets_equal_oracle(name):
         assert np.array_equal(goff, off) and np.array_equal(gadj, adj)
 
 
+@pytest.mark.parametrize("n", [64 * (2**20 - 1), 64 * (2**20 - 1) + 1])
+def test_most_buckets_and_one_more_row(n):
+    """Just under 2^26 rows there are 2^20 - 1 buckets of 64 rows, the most; from
+    the next row on all entries are sorted at once."""
+    import paper_2509_02590_gb300 as wcc
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    u, v = _random(n, 200_000, 40)
+    u[:5], v[:5] = [n - 1, n - 2, n - 1, 0, n - 65], [n - 2, n - 1, 0, n - 1, n - 1]
+    u[5:3000] = n - 1 - u[5:3000] % 130  # the last buckets are not empty
+    src, dst = u.astype(np.int32), v.astype(np.int32)
+    off, adj = oracle.build_csr(n, src, dst)
+    with wcc.WccGraph.from_edges(torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda(), n) as g:
+        goff, gadj = g.csr()
+    assert np.array_equal(goff, off) and np.array_equal(gadj, adj)
+
+
 def _copies_of_one_edge(extra):
     """2^30 + extra edges on 900,000 vertices, all but 5,000 of them 0-1: more
     than 2^31 entries in the first bucket, which holds rows 0 and 1.  Run in a
