@@ -1063,8 +1063,8 @@ int wcc_number_by_minima(const int32_t *minima, int64_t n, int32_t *labels_out, 
       o = static_cast<int32_t *>(dout.ensure(4 * n));
     }
     check_minima(mn, n, ws, s);
-    unsigned *werr = n > 0 ? number_clusters(mn, n, o, ws, s) : nullptr;
-    if (werr && read_back(werr, s)) check_device_error(DERR_TIMEOUT, "numbering");
+    unsigned *werr = n > 0 ? number_clusters(mn, n, o, ws, s) : nullptr, herr = 0;
+    if (werr) WCC_CUDA(cudaMemcpyAsync(&herr, werr, 4, cudaMemcpyDeviceToHost, s));
     int32_t top = -1;
     if (n > 0) {
       // ids are dense and ascending by smallest vertex: K = 1 + the largest id
@@ -1073,8 +1073,12 @@ int wcc_number_by_minima(const int32_t *minima, int64_t n, int32_t *labels_out, 
       k_max_i32_launch(o, n, mx, s);
       WCC_CUDA(cudaMemcpyAsync(&top, mx, 4, cudaMemcpyDeviceToHost, s));
     }
-    if (!on_device && n > 0) WCC_CUDA(cudaMemcpyAsync(labels_out, o, 4 * n, cudaMemcpyDeviceToHost, s));
-    WCC_CUDA(cudaStreamSynchronize(s));
+    WCC_CUDA(cudaStreamSynchronize(s));  // one wait for the error word and the result
+    if (herr) check_device_error(DERR_TIMEOUT, "numbering");
+    if (!on_device && n > 0) {
+      WCC_CUDA(cudaMemcpyAsync(labels_out, o, 4 * n, cudaMemcpyDeviceToHost, s));
+      WCC_CUDA(cudaStreamSynchronize(s));
+    }
     if (k) *k = (int64_t)top + 1;
   });
 }

@@ -225,10 +225,14 @@ void job_finish(Job *j, int32_t *out, int on_device, cudaStream_t s, wcc_stats *
   int32_t *d_out = out;
   if (!on_device) d_out = static_cast<int32_t *>(j->out.ensure(4 * (size_t)j->n));
   unsigned *err = number_clusters(j->lmin.as<int32_t>(), j->n, d_out, j->g->ws, s);
-  if (err && read_back(err, s)) check_device_error(DERR_TIMEOUT, "numbering");
-  if (!on_device)
+  unsigned herr = 0;
+  if (err) WCC_CUDA(cudaMemcpyAsync(&herr, err, 4, cudaMemcpyDeviceToHost, s));
+  const ReqCtx h = read_back(j->req.as<ReqCtx>(), s);  // one wait for both
+  if (herr) check_device_error(DERR_TIMEOUT, "numbering");
+  if (!on_device) {
     WCC_CUDA(cudaMemcpyAsync(out, d_out, 4 * (size_t)j->n, cudaMemcpyDeviceToHost, s));
-  const ReqCtx h = read_back(j->req.as<ReqCtx>(), s);
+    WCC_CUDA(cudaStreamSynchronize(s));
+  }
   if (stats) {
     stats->in_clusters = j->in_clusters;
     stats->out_clusters = h.accepted;
