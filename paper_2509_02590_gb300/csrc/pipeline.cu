@@ -57,31 +57,38 @@ __global__ void k_make_keys(const int32_t *__restrict__ lab, int64_t n, uint32_t
 
 // ---- single-pass running counts over tiles -----------------------------------
 // A tile's status word: 2 bits of state (its own count, or the count up to its
-// end), 62 of value.  Thread 0 of the tile's block calls; returns the count of
-// all earlier tiles.  Tiles are handed out in order, so every wait ends; one
-// that outlasts a second sets DERR_TIMEOUT.
+// end), 62 of value.  Warp 0 of the tile's block calls; returns the count of all
+// earlier tiles, 32 of them at a look.  Tiles are handed out in order, so every
+// wait ends; one that outlasts a second sets DERR_TIMEOUT.
+// (One thread walking back tile by tile takes as long as the tiles in flight are
+// many: numbering 1M vertices 0.094 ms a call instead of 0.080, 100M 1.65 instead of
+// 1.36; grouping 10M 1.09 instead of 1.03.)
 constexpr unsigned long long TS_OWN = 1ull << 62, TS_ALL = 2ull << 62, TS_VAL = (1ull << 62) - 1;
 __device__ __forceinline__ unsigned long long tiles_before(unsigned long long *status, int64_t tile,
                                                            unsigned long long own, unsigned *err) {
+  const int lane = threadIdx.x & 31;
   unsigned long long before = 0;
   if (tile > 0) {
-    atomicExch(&status[tile], TS_OWN | own);
+    if (lane == 0) atomicExch(&status[tile], TS_OWN | own);
     const uint64_t t0 = globaltimer_ns();
     for (int64_t p = tile - 1; p >= 0;) {
-      const unsigned long long w = *(volatile unsigned long long *)&status[p];
-      if ((w >> 62) == 0) {
-        if (globaltimer_ns() - t0 > 1000ull * 1000 * 1000) {
-          atomicOr(err, DERR_TIMEOUT);
-          break;
-        }
-        continue;
+      unsigned long long w = TS_ALL;  // before the first tile: nothing
+      if (p - lane >= 0) w = *(volatile unsigned long long *)&status[p - lane];
+      const unsigned ready = __ballot_sync(FULL, (w >> 62) != 0);
+      const unsigned all = __ballot_sync(FULL, (w >> 62) == 2ull);
+      // the tiles up to the first with a count from the start, as far as they have one
+      const int ends = all ? __ffs(all) : 33, gap = ready == FULL ? 32 : __ffs(~ready) - 1;
+      const int use = min(ends, gap);
+      before += warp_sum(lane < use ? w & TS_VAL : 0ull);
+      if (use == ends) break;
+      p -= use;
+      if (use == 0 && globaltimer_ns() - t0 > 1000ull * 1000 * 1000) {
+        if (lane == 0) atomicOr(err, DERR_TIMEOUT);
+        break;
       }
-      before += w & TS_VAL;
-      if ((w >> 62) == 2ull) break;
-      --p;
     }
   }
-  atomicExch(&status[tile], TS_ALL | (before + own));
+  if (lane == 0) atomicExch(&status[tile], TS_ALL | (before + own));
   return before;
 }
 
@@ -128,7 +135,10 @@ __global__ void __launch_bounds__(TB) k_clusters(const uint32_t *__restrict__ sk
   }
   int tot;
   const int ex = block_exclusive_scan<TB>(heads, &tot, sm);
-  if (threadIdx.x == 0) before_sh = tiles_before(status, tile, (unsigned long long)tot, &info->err);
+  if (threadIdx.x < 32) {
+    const unsigned long long b = tiles_before(status, tile, (unsigned long long)tot, &info->err);
+    if (threadIdx.x == 0) before_sh = b;
+  }
   __syncthreads();
   int64_t c = (int64_t)before_sh + ex - 1;  // the cluster the thread's first position continues
   const int64_t c0 = c + ((first & 1u) ? 1 : 0);
@@ -448,7 +458,10 @@ __global__ void __launch_bounds__(TB) k_rank(const int32_t *__restrict__ lmin, i
   for (int z = 0; z < CI; ++z) mine += base + z < n && l[z] == (int32_t)(base + z);
   int tot;
   const int ex = block_exclusive_scan<TB>(mine, &tot, sm);
-  if (threadIdx.x == 0) before_sh = tiles_before(status, tile, (unsigned long long)tot, err);
+  if (threadIdx.x < 32) {
+    const unsigned long long b = tiles_before(status, tile, (unsigned long long)tot, err);
+    if (threadIdx.x == 0) before_sh = b;
+  }
   __syncthreads();
   uint32_t r = (uint32_t)before_sh + (uint32_t)ex;
 #pragma unroll

@@ -91,3 +91,50 @@ def test_device_output_that_only_a_copy_can_write(n):
 @pytest.mark.parametrize("kind", ["none", "one", "distinct", "pairs", "mixed"])
 def test_sizes_around_the_one_cta_limit(n, kind):
     test_sizes(n, kind)
+
+
+@pytest.mark.parametrize("tiles", [32, 33, 34, 64, 65, 66, 500])
+@pytest.mark.parametrize("over", [-1, 0, 1])
+def test_running_counts_over_many_tiles(tiles, over):
+    """The single-pass counts look back over 32 tiles of 2,048 positions at a
+    time: numbering (representatives before a vertex) and grouping (clusters
+    before a sorted position) at and around those sizes, with tiles that count
+    nothing among them."""
+    import paper_2509_02590_gb300 as wcc
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    n = 2048 * tiles + over
+    rng = np.random.default_rng(n)
+    v = np.arange(n)
+    width = np.where(rng.random(n) < 0.5, 1, 5000)  # runs of one vertex, and longer than two tiles
+    minima = np.zeros(n, np.int64)
+    at = 0
+    for w in width:
+        if at >= n:
+            break
+        minima[at:at + w] = at
+        at += w
+    ref = np.cumsum(minima == v) - 1
+    ids, k = torch.empty(n, dtype=torch.int32, device="cuda"), None
+    mn = torch.from_numpy(minima.astype(np.int32)).cuda()
+    k = wcc._binding.wcc_number_by_minima(mn.data_ptr(), n, ids.data_ptr(), 1,
+                                          torch.cuda.current_stream().cuda_stream)
+    want = ref[minima]
+    assert k == int(ref[-1]) + 1 and np.array_equal(ids.cpu().numpy(), want)
+    # the same runs as input clusters, joined up as paths: components in, components out
+    same = np.nonzero(minima[1:] == minima[:-1])[0]
+    perm = rng.permutation(n)
+    src, dst = perm[same].astype(np.int32), perm[same + 1].astype(np.int32)
+    lab = np.empty(n, np.int32)
+    lab[perm] = minima
+    with wcc.WccGraph.from_edges(torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda(), n) as g:
+        out, st = g.run(torch.from_numpy(lab).cuda(), rule="linear", num=0, den=1, stats=True)
+    assert st["in_clusters"] == k
+    sizes = np.bincount(want)
+    low = np.full(k, n)
+    np.minimum.at(low, want, perm)
+    order = np.argsort(low[sizes > 1])
+    rank = np.full(k, -1)
+    rank[np.nonzero(sizes > 1)[0][order]] = np.arange(len(order))
+    got = out.cpu().numpy()
+    assert np.array_equal(got[perm], rank[want])
