@@ -33,10 +33,10 @@
 //
 // Measured (builds with L2 flushed, before: rows by global atomics up to 2^24
 // edges, one radix sort of 64-bit keys above): 172M edges on 10M vertices
-// 23.5 -> 9.1 ms, 53M on 3M 7.4 -> 2.6 ms, 11.7M raw on 1M 1.69 -> 0.82 ms,
+// 23.5 -> 9.1 ms, 53M on 3M 7.4 -> 2.5 ms, 11.7M raw on 1M 1.69 -> 0.78 ms,
 // 0.9M on 100,000 0.197 -> 0.136 ms, 21,000 on 2,000 0.110 -> 0.111 ms.  On the
-// 3M-vertex graph the bucket sort takes 1.17 ms (107M entries, 3.4 cycles an
-// entry and SM: shuffles and shared-memory atomics), the two partitions 0.86
+// 3M-vertex graph the bucket sort takes 1.09 ms (107M entries, 3.2 cycles an
+// entry and SM: shuffles and shared-memory atomics), the two partitions 0.85
 // (2.6 GB moved, 3 TB/s: ranking bounds it), the counts 0.30.
 #include <algorithm>
 
