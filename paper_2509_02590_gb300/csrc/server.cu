@@ -96,10 +96,11 @@ size_t estimate_bytes(int64_t n) { return (size_t)n * 240 + (1u << 20); }
 size_t graph_bytes(int64_t n, int64_t m) { return 2 * (8 * (size_t)(n + 1) + 8 * (size_t)m); }
 
 // The builder's transient memory while one such graph is built (the edge
-// copies and, by buckets, one 64-bit and one 32-bit entry array over the 2m
-// directed entries; by the radix sort, two 64-bit key arrays, two 32-bit flag
-// arrays, scan and sort temporaries: the larger), rounded up: needed only
-// during the admission that builds it.
+// copies and, over the 2m directed entries, two 64-bit key arrays, two 32-bit flag
+// arrays, scan and sort temporaries for the radix sort, and no more by buckets:
+// one 64-bit and one 32-bit array, and as many again at most for the entries of
+// large buckets that are left to the radix sort), rounded up: needed only during
+// the admission that builds it.
 size_t build_bytes(int64_t n, int64_t m) { return 2 * (56 * (size_t)m + 8 * (size_t)n) + (1u << 20); }
 
 struct Server {
@@ -445,6 +446,8 @@ uint64_t submit(Server *S, Graph *g, const int32_t *src, const int32_t *dst, int
   R->n = n;
   R->rule = checked_rule(rule);
   R->min_size = min_size < 2 ? 2 : min_size;
+  // an unclaimed queue index stands for an item of at least two vertices, and no
+  // two items share one (a part that its CTA keeps has no index of its own)
   R->ring_need = n / 2 + 2;
   if ((int64_t)(R->est_bytes + R->build_bytes) > S->budget)
     fail(WCC_ERR_BUSY, "a graph of " + std::to_string(n) + " vertices and " + std::to_string(m) +
