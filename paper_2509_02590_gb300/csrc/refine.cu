@@ -272,6 +272,13 @@ __device__ __forceinline__ int uf_find(int32_t *p, int x) {
   return x;
 }
 
+// The same without writing.
+__device__ __forceinline__ int uf_root(const int32_t *p, int x) {
+  const volatile int32_t *vp = p;
+  for (int y; (y = vp[x]) != x;) x = y;
+  return x;
+}
+
 __device__ __forceinline__ void uf_union(int32_t *p, int a, int b) {
   for (;;) {
     a = uf_find(p, a);
@@ -387,8 +394,11 @@ __device__ __forceinline__ void afforest(const Mem<IT> &m, int n, int32_t *uf, i
     }
   }
   __syncthreads();
+  // the roots, by walks that write nothing on their way: a walk that halves its
+  // path could store an ancestor over a root that another thread has just written,
+  // and leave that vertex a component of its own
   for (int i = threadIdx.x; i < n; i += RB)
-    if (m.alive[i]) uf[i] = uf_find(uf, i);
+    if (m.alive[i]) uf[i] = uf_root(uf, i);
   __syncthreads();
 }
 

@@ -310,3 +310,29 @@ def test_statistics_of_batches_of_small_items(wcc):
             out, st = g.run(lab_dev, min_size=w.min_size, stats=True)
             assert {k: st[k] for k in want} == want
     assert np.array_equal(out.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("trees", [20, 40])
+def test_components_by_union_find_every_time(wcc, trees):
+    """Clusters of 20 and of 40 random trees of 40 vertices (left to the
+    union-find after 32 thin rounds and after 32 components).  Its chains are
+    several links long when the roots are written at its end, and a vertex left
+    with another ancestor would be a component of its own: 400 such clusters, 100
+    runs, T = 0, so the components are the output."""
+    rng = np.random.default_rng(3)
+    eu, ev, lab, n = [], [], [], 0
+    for c in range(400):
+        for _ in range(trees):
+            i = np.arange(1, 40)
+            eu.append(n + i); ev.append(n + (rng.random(39) * i).astype(np.int64))
+            lab.append(np.full(40, c))
+            n += 40
+    w = _finish(rng, n, np.concatenate(eu), np.concatenate(ev), np.concatenate(lab), 2, "trees")
+    off, adj = oracle.build_csr(w.n, w.src, w.dst)
+    ref, _ = oracle.wcc(w.n, off, adj, w.labels, 2, kind=oracle.RULE_LINEAR, num=0, den=1)
+    assert ref.max() + 1 == 400 * trees
+    lab_dev, want = torch.from_numpy(w.labels).cuda(), torch.from_numpy(ref).cuda()
+    with wcc.WccGraph.from_edges(w.src, w.dst, w.n) as g:
+        wrong = sum(not torch.equal(g.run(lab_dev, rule="linear", num=0, den=1), want)
+                    for _ in range(100))
+    assert wrong == 0
